@@ -118,7 +118,13 @@ typedef struct {
  *   finds faster; banks of one or two spindowns run blocks of 4 neighbouring
  *   sky points (consecutive ones of the bank, or of a neighbour order of its
  *   sky list) sharing one staged window; else FARPOLY where it applies, else
- *   DIRECT.  Results do not depend on the grouping. */
+ *   DIRECT.  Results of these forms do not depend on the grouping.
+ *   Large banks of dense sky lists (column steps P df T = 1 bin, uniform
+ *   spindowns, no coverage, no tile request) run the direct sum on the tensor
+ *   cores instead where the planner finds that faster: window sums from FP16
+ *   pairs of bins and weights with FP32 accumulation, closer to the exact sum
+ *   than SINCPOLY; in the last bits its results depend on which sky points
+ *   share a tile, so on the sky list. */
 typedef enum {
     FSTAT_ALGO_AUTO = 0,
     FSTAT_ALGO_DIRECT = 1,
@@ -308,6 +314,13 @@ int fstat_test_ring_stall(fstat_ctx *ctx, int32_t after_sft);
  *           118 and 119 the sinc form for L = 1 banks (P = 8); 107 and up use
  *           the TMA-ring staging). */
 int fstat_get_plan(fstat_ctx *ctx, int32_t *out);
+
+/* Inspection: the tiles of the tensor-core form (see AUTO) the current bank
+ * runs in, out[4] = (rows per tile, row tiles, column blocks, groups of 16 bin
+ * positions a tile's windows span at most), or all 0 where it does not run;
+ * fstat_get_plan then describes the kernel that it replaces.
+ * Errors: as fstat_get_plan. */
+int fstat_get_tensor_tiles(fstat_ctx *ctx, int32_t *out);
 
 /* Number of CUDA kernels this context has launched since it was created. */
 int fstat_get_launch_count(fstat_ctx *ctx, int64_t *n_launches);

@@ -76,6 +76,7 @@ SIGNATURES = {
     "fstat_get_bins": (ctypes.c_int, [_P, _I32, _P, _I32]),
     "fstat_get_error_flags": (ctypes.c_int, [_P, ctypes.POINTER(_I32)]),
     "fstat_get_plan": (ctypes.c_int, [_P, _P]),
+    "fstat_get_tensor_tiles": (ctypes.c_int, [_P, _P]),
     "fstat_test_ring_stall": (ctypes.c_int, [_P, _I32]),
     "fstat_set_noise_floor": (ctypes.c_int, [_P, _I32]),
     "fstat_set_coverage": (ctypes.c_int, [_P, _P, _P, _I32]),
@@ -291,6 +292,13 @@ def fstat_get_plan(ctx) -> dict:
     _check(ctx, _lib.fstat_get_plan(ctx, _host_ptr(out)))
     keys = ("P", "L", "M", "warps", "sft_chunk", "lg_row", "w_pairs", "variant")
     return {k: int(v) for k, v in zip(keys, out)}
+
+
+def fstat_get_tensor_tiles(ctx) -> dict:
+    """Tiles of the tensor-core form for the current bank (all 0: another form runs)."""
+    out = np.zeros(4, dtype=np.int32)
+    _check(ctx, _lib.fstat_get_tensor_tiles(ctx, _host_ptr(out)))
+    return {k: int(v) for k, v in zip(("rows", "tiles", "column_blocks", "groups"), out)}
 
 
 def fstat_get_launch_count(ctx) -> int:
@@ -583,6 +591,9 @@ class FStat:
 
     def plan(self) -> dict:
         return fstat_get_plan(self.ctx)
+
+    def tensor_tiles(self) -> dict:
+        return fstat_get_tensor_tiles(self.ctx)
 
     def take_kernel_time(self):
         return fstat_take_kernel_time(self.ctx)

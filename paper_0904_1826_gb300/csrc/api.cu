@@ -85,6 +85,12 @@ struct Plan {
     bool two = false;   // two-row tiles of the sinc ring form (L = 2)
     int sky_rows = 1;   // sky points per block of the one-row ring (meta and bases SFT-major when > 1)
     bool sky_perm = false;   // blocks group the sky points in the context's neighbour order
+    // tensor-core form (dirichlet_tc.cu) of this bank; the fields above stay
+    // the ring plan it replaces (reported by fstat_get_plan)
+    bool tc = false;
+    bool tc_perm = false;    // tiles take the sky points in tc_order
+    int tc_sub = 1, tc_rt = kTcRows, tc_tiles = 0, tc_colb = 0;   // templates per bin, rows per tile, tiles, column blocks
+    int tc_gk = 4;           // groups of 16 positions the windows of a tile span at most
     size_t smem = 0;
     long long grid = 0;
 };
@@ -160,9 +166,18 @@ struct fstat_ctx {
     bool batch_member = false;        // a workunit of a batch (kernels with a persistent form only)
     std::vector<int> h_order;         // sky points in neighbour order (empty: not computed yet)
     double order_spread4 = -1.0;      // window spread bound of 4 consecutive points of h_order (bins)
-    int* d_perm = nullptr;            // [n_sky] h_order on the device
-    int* d_rank = nullptr;            // [n_sky] each sky point's place in h_order
-    bool perm_on_device = false;
+    std::vector<int> tc_order;        // neighbour order for the tensor-core form's tiles
+    int* d_perm = nullptr;            // [n_sky] h_order or tc_order on the device
+    int* d_rank = nullptr;            // [n_sky] each sky point's place in that order
+    int perm_on_device = 0;           // 0: none, 1: h_order, 2: tc_order
+    // tensor-core form: tables, their extent, and the blocks' scratch
+    unsigned char* d_gtab = nullptr;
+    float* d_inv = nullptr;
+    float4* d_tcs = nullptr;
+    size_t cap_gtab = 0, cap_inv = 0, cap_tcs = 0;
+    int gt_nblk = -1, gt_xoff = -1;
+    bool gt_dirty = true;
+    fstat_opts opts0{};               // the options as created (the autotuner changes opts)
     double dfdot = 0.0;
     // derived per-bank buffers
     size_t cap_meta = 0, cap_kh0 = 0, cap_ph0 = 0, cap_abcd = 0, cap_comb = 0, cap_twoF = 0;
@@ -395,6 +410,140 @@ SincGamma sinc_gamma() {
         }
     }
     return G;
+}
+
+// Bound, in bins, on how far apart the windows of a tile's rows can start
+// (tensor-core form): rows are (sky place, spindown, sub-bin offset) in
+// grouping order, rt rows a tile.  Two sky points' khat differ by at most
+// f_max T 1.1e-4 |n_1 - n_2| and |n_1 - n_2| <= 2 max |n - mean n| over the
+// tile; the spindowns spread it by |fdot range| tau T, the offsets by less
+// than a bin.
+double tc_spread_bins(const fstat_ctx* c, const std::vector<double>& unit, int rps, int rt, const std::vector<int>* order) {
+    const double k_max = (c->f0 + (c->n_f - 1) * c->df) * c->T;
+    double r_max = 0.0;
+    const long long n_rows = (long long)c->n_sky * rps;
+    for (long long g0 = 0; g0 < n_rows; g0 += rt) {
+        const int a = (int)(g0 / rps), b = (int)((std::min(n_rows, g0 + rt) - 1) / rps);
+        double m[3] = {0, 0, 0};
+        for (int i = a; i <= b; ++i)
+            for (int k = 0; k < 3; ++k) m[k] += unit[3 * (order ? (*order)[i] : i) + k];
+        for (int k = 0; k < 3; ++k) m[k] /= b - a + 1;
+        for (int i = a; i <= b; ++i) {
+            const double* u = &unit[3 * (order ? (*order)[i] : i)];
+            const double q = (u[0] - m[0]) * (u[0] - m[0]) + (u[1] - m[1]) * (u[1] - m[1]) + (u[2] - m[2]) * (u[2] - m[2]);
+            r_max = std::max(r_max, q);
+        }
+    }
+    double fd_min = c->h_fdot[0], fd_max = c->h_fdot[0], tau = 0.0;
+    for (double v : c->h_fdot) {
+        fd_min = std::min(fd_min, v);
+        fd_max = std::max(fd_max, v);
+    }
+    for (int d = 0; d < kMaxDet; ++d)
+        for (double t : c->det[d].t_start) tau = std::max(tau, std::fabs(t + 0.5 * c->T - c->t_ref));
+    return k_max * 1.1e-4 * 2.0 * std::sqrt(r_max) + (fd_max - fd_min) * (tau + 500.0) * c->T * 1.00011 + 2.0;
+}
+
+// Sky points in bands of delta, alpha back and forth, for tiles of g
+// consecutive points (a square patch of g of n points is side = sqrt(4 pi g /
+// n) wide).  by_count = false: bands of equal width in delta, about `side`.
+// true: from the south pole up, each band takes the points of as many whole
+// tiles as its circumference has sides, which follows the density of the list
+// and leaves no tile across two bands.  Largest distance of a point from its
+// tile's mean, lattice skies, tiles of 128 rows (equal width / by count):
+// 3001 points of one spindown 1.09 / 0.58, 20 000 0.43 / 0.23, 4000 of ten
+// 0.28 / 0.22, 1500 of seven 0.45 / 0.57.
+std::vector<int> tc_neighbour_order(const fstat_ctx* c, double g, bool by_count) {
+    const int n = c->n_sky;
+    const double side = std::sqrt(4.0 * kPi * std::max(1.0, g) / n);
+    std::vector<double> alpha(n);
+    for (int i = 0; i < n; ++i) {
+        alpha[i] = std::fmod(c->h_sky[2 * i], 2.0 * kPi);
+        if (alpha[i] < 0) alpha[i] += 2.0 * kPi;
+    }
+    std::vector<int> order(n);
+    for (int i = 0; i < n; ++i) order[i] = i;
+    auto delta = [&](int i) { return c->h_sky[2 * (size_t)i + 1]; };
+    std::sort(order.begin(), order.end(), [&](int x, int y) { return delta(x) < delta(y) || (delta(x) == delta(y) && x < y); });
+    const double width = kPi / std::max(1.0, std::round(kPi / side));
+    bool back = false;
+    for (int i = 0; i < n; back = !back) {
+        int m = 0;
+        if (by_count) {
+            const double mid = std::min(delta(order[i]) + 0.5 * side, 0.5 * kPi);
+            m = (int)std::min<double>(n - i, std::round(g * std::max(1.0, std::round(2.0 * kPi * std::cos(mid) / side))));
+            if (m < 1 || n - i - m < 0.5 * g) m = n - i;
+        } else {
+            const double b = std::floor((delta(order[i]) + 0.5 * kPi) / width);
+            while (i + m < n && (m == 0 || std::floor((delta(order[i + m]) + 0.5 * kPi) / width) == b)) ++m;
+        }
+        std::sort(order.begin() + i, order.begin() + i + m, [&](int x, int y) {
+            if (alpha[x] != alpha[y]) return back ? alpha[x] > alpha[y] : alpha[x] < alpha[y];
+            return x < y;
+        });
+        i += m;
+    }
+    return order;
+}
+
+// Tensor-core form where it is the faster one.  It needs column steps of one
+// bin (n_sub = P / L templates a bin), a uniform spindown grid, at least 8 SFTs
+// (its blocks work up to 6 ahead) and windows of a tile's rows within
+// kTcMaxSpread bins; frequency coverage, Kahan sums, other D and explicit tile
+// or form requests keep the other forms.
+void choose_tc(fstat_ctx* c, int P, int L, bool found, Plan& pl) {
+    pl.tc = false;
+    const fstat_opts& o = c->opts0;
+    if (!found || P % L != 0 || !c->fdot_uniform || c->have_cov || c->n_sft < 8) return;
+    if (o.algo != FSTAT_ALGO_AUTO || o.tile_m > 0 || o.tile_warps > 0 || o.sft_chunk > 0) return;
+    const int n_sub = P / L, rps = c->n_fdot * n_sub;
+    const long long n_rows = (long long)c->n_sky * rps;
+    const long long n_col = (c->n_f + n_sub - 1) / n_sub;
+    const long long colb = (n_col + kTcCols - 1) / kTcCols;
+    const int sms = current_sm_count();
+    // Measured on GB300: a block takes 1.44 us an SFT for a tile of 128 x 64
+    // templates, whatever part of it is filled; the other forms 5.6e11 pairs/s on
+    // large banks of three or more spindowns, 4.6e11 on one or two, and 2.7e11
+    // where the steps are 1/8 bin (L = 1); smaller banks leave them slower.
+    auto t_tc = [&](int rt) {
+        const long long items = ((n_rows + rt - 1) / rt) * colb;
+        return (double)((items + sms - 1) / sms) * c->n_sft * 1.44e-6;
+    };
+    const double rate = L == 1 ? 2.7e11 : c->n_fdot <= 2 ? 4.6e11 : 5.6e11;
+    const double t_other = (double)c->n_sky * c->n_fdot * c->n_f * c->n_sft / rate;
+    if (n_rows > (1 << 28) || (n_rows / 32 + 1) * colb > (1 << 28) || t_other > 3000.0) return;   // 32-bit counters
+    if (t_tc(kTcRows) > 0.92 * t_other) return;
+    std::vector<double> unit(3 * (size_t)c->n_sky);
+    for (int i = 0; i < c->n_sky; ++i) {
+        const double al = c->h_sky[2 * i], de = c->h_sky[2 * i + 1];
+        unit[3 * i] = std::cos(de) * std::cos(al);
+        unit[3 * i + 1] = std::cos(de) * std::sin(al);
+        unit[3 * i + 2] = std::sin(de);
+    }
+    for (int rt = kTcRows; rt >= 32 && t_tc(rt) <= 0.92 * t_other; rt /= 2) {
+        double spread = tc_spread_bins(c, unit, rps, rt, nullptr);
+        bool nat = true;
+        c->perm_on_device = 0;
+        for (const bool by_count : {false, true}) {
+            std::vector<int> order = tc_neighbour_order(c, (double)rt / rps, by_count);
+            const double q = tc_spread_bins(c, unit, rps, rt, &order);
+            if (q < spread) {
+                spread = q;
+                nat = false;
+                c->tc_order = std::move(order);
+            }
+        }
+        if (spread > kTcMaxSpread) continue;
+        pl.tc = true;
+        pl.tc_perm = !nat;
+        pl.tc_sub = n_sub;
+        pl.tc_rt = rt;
+        pl.tc_tiles = (int)((n_rows + rt - 1) / rt);
+        pl.tc_colb = (int)colb;
+        // a window starts up to 3 positions into its first block
+        pl.tc_gk = std::max(2, std::min(4, (int)std::ceil((spread + 3.0 + 16.0) / 16.0)));
+        return;
+    }
 }
 
 bool far_eligible(const fstat_ctx* c) {
@@ -839,7 +988,10 @@ int make_plan(fstat_ctx* c, Plan& out) {
                 }
     }
     if (far_eligible(c)) {
-        if (make_far_plan(c, P, L, found, out)) return FSTAT_OK;
+        if (make_far_plan(c, P, L, found, out)) {
+            choose_tc(c, P, L, found, out);
+            return FSTAT_OK;
+        }
         if (c->opts.algo == FSTAT_ALGO_FARPOLY)
             return fail(c, FSTAT_EINVAL, "no far-field tile plan fits this template bank");
     }
@@ -1039,6 +1191,7 @@ int refresh_sft_state(fstat_ctx* c, cudaStream_t s) {
     CUDA_TRY(c, cudaStreamSynchronize(s));
     c->sft_dirty = false;
     c->tab_dirty = true;
+    c->gt_dirty = true;
     return FSTAT_OK;
 }
 
@@ -1071,6 +1224,7 @@ int fstat_create(fstat_ctx** out, int device, const fstat_opts* opts) {
     fstat_ctx* c = new fstat_ctx();
     c->device = device;
     c->opts = o;
+    c->opts0 = o;
     c->gam = far_gamma();
     c->sgam = sinc_gamma();
     if (set_device(c) != FSTAT_OK) {
@@ -1109,7 +1263,7 @@ void fstat_destroy(fstat_ctx* c) {
                     c->tw.hist, c->tw.state, c->tw.tie_count, c->tw.cand_idx, c->tw.cand_val, c->tw.n_cand,
                     c->tw.out_idx, c->tw.out_val, c->d_inj_work, c->d_sig, c->d_ptab, c->d_pcoef,
                     c->d_bins_w, c->d_floor, c->d_sbar, c->d_weight, c->d_cov, c->d_comb_j, c->d_slide_seg, c->d_slide_A,
-                    c->d_slide_B, c->d_slide_out, c->d_perm, c->d_rank};
+                    c->d_slide_B, c->d_slide_out, c->d_perm, c->d_rank, c->d_gtab, c->d_inv, c->d_tcs};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (int i = 0; i < kTimedRing; ++i) {
@@ -1340,8 +1494,9 @@ int fstat_set_templates(fstat_ctx* c, const double* sky, int32_t n_sky, double f
     c->h_sky.assign(sky, sky + 2 * (size_t)n_sky);
     c->h_fdot.assign(fdot, fdot + n_fdot);
     c->h_order.clear();
+    c->tc_order.clear();
     c->order_spread4 = -1.0;
-    c->perm_on_device = false;
+    c->perm_on_device = 0;
     if (c->d_sky) cudaFree(c->d_sky);
     if (c->d_fdot) cudaFree(c->d_fdot);
     c->d_sky = nullptr;
@@ -1406,18 +1561,45 @@ int prepare(fstat_ctx* c, cudaStream_t s) {
 // follow the plan (form, window width), so a new plan may need a rebuild.
 int ensure_tables(fstat_ctx* c, cudaStream_t s) {
     int rc;
-    if (c->plan.sky_perm && !c->perm_on_device) {   // the neighbour order and its inverse
+    const int want_perm = c->plan.tc ? (c->plan.tc_perm ? 2 : 0) : (c->plan.sky_perm ? 1 : 0);
+    if (want_perm && c->perm_on_device != want_perm) {   // the neighbour order and its inverse
+        const std::vector<int>& order = want_perm == 2 ? c->tc_order : c->h_order;
         const int n = c->n_sky;
         std::vector<int> rank(n);
-        for (int i = 0; i < n; ++i) rank[c->h_order[i]] = i;
+        for (int i = 0; i < n; ++i) rank[order[i]] = i;
         if (c->d_perm) cudaFree(c->d_perm);
         if (c->d_rank) cudaFree(c->d_rank);
         c->d_perm = c->d_rank = nullptr;
         CUDA_TRY(c, cudaMalloc(&c->d_perm, (size_t)n * sizeof(int)));
         CUDA_TRY(c, cudaMalloc(&c->d_rank, (size_t)n * sizeof(int)));
-        CUDA_TRY(c, cudaMemcpy(c->d_perm, c->h_order.data(), (size_t)n * sizeof(int), cudaMemcpyHostToDevice));
+        CUDA_TRY(c, cudaMemcpy(c->d_perm, order.data(), (size_t)n * sizeof(int), cudaMemcpyHostToDevice));
         CUDA_TRY(c, cudaMemcpy(c->d_rank, rank.data(), (size_t)n * sizeof(int), cudaMemcpyHostToDevice));
-        c->perm_on_device = true;
+        c->perm_on_device = want_perm;
+    }
+    if (c->plan.tc) {
+        // positions reach from the lowest window of the bank, rounded down to a
+        // block, to the widest tile window above the highest one (whose columns
+        // run up to a column block past the band)
+        int xoff = 0, n_pos = 0;
+        far_extent(c, kTcCols + 4 * kTcBlkMax + 8, &xoff, &n_pos);
+        xoff = (xoff + 4 + 3) & ~3;
+        const int n_blk = (n_pos + 8 + 3) / 4;
+        if ((rc = grow(c, &c->d_tcs, c->cap_tcs,
+                       (size_t)std::min(c->plan.tc_tiles * c->plan.tc_colb, current_sm_count()) * 2 * kTcRows * kTcCols)) !=
+            FSTAT_OK)
+            return rc;
+        if (c->gt_dirty || c->gt_nblk != n_blk || c->gt_xoff != xoff) {
+            if ((rc = grow(c, &c->d_gtab, c->cap_gtab, (size_t)c->n_sft * n_blk * 256)) != FSTAT_OK) return rc;
+            if ((rc = grow(c, &c->d_inv, c->cap_inv, (size_t)c->n_sft)) != FSTAT_OK) return rc;
+            const void* bins = c->opts.bins_form == FSTAT_BINS_C64 ? (const void*)work_bins(c) : (const void*)c->d_bins16;
+            CUDA_TRY(c, launch_tc_tables(bins, c->opts.bins_form, c->row, c->n_sft, c->n_bins, n_blk, xoff, c->d_gtab,
+                                         c->d_inv, s));
+            c->launches += 1;
+            c->gt_dirty = false;
+            c->gt_nblk = n_blk;
+            c->gt_xoff = xoff;
+        }
+        return FSTAT_OK;
     }
     if (c->plan.far) far_extent(c, c->plan.w_pairs, &c->far_xoff, &c->n_pos);
     if (c->plan.far &&
@@ -1469,6 +1651,14 @@ TimingParams timing_params(const fstat_ctx* c, int n_sky) {
     tp.sft_major = c->plan.sky_rows > 1 ? 1 : 0;   // blocks of several sky points read them SFT-major
     tp.sky_rank = c->plan.sky_perm ? c->d_rank : nullptr;
     tp.row_rot = (c->plan.rows || c->plan.two) ? 1 : 0;   // the row-tiled forms step the twiddle across rows
+    if (c->plan.tc) {   // drift and twiddle step over 4 columns of a bin each
+        tp.P = 4 * c->plan.tc_sub;
+        tp.L = 4;
+        tp.M = 1;
+        tp.sft_major = 1;
+        tp.sky_rank = c->plan.tc_perm ? c->d_rank : nullptr;
+        tp.row_rot = 0;
+    }
     tp.kh0 = c->fdot_uniform ? nullptr : c->d_kh0;
     tp.ph0 = c->fdot_uniform ? nullptr : c->d_ph0;
     tp.abcd = c->d_abcd;
@@ -1517,6 +1707,35 @@ DirichletParams dirichlet_params(const fstat_ctx* c) {
     return dp;
 }
 
+TcParams tc_params(const fstat_ctx* c) {
+    const Plan& pl = c->plan;
+    TcParams t{};
+    t.gtab = c->d_gtab;
+    t.inv_scale = c->d_inv;
+    t.n_blk = c->gt_nblk;
+    t.xoff = c->gt_xoff;
+    t.k_lo = c->k_lo;
+    t.meta = c->d_meta;
+    t.base = c->d_base;
+    t.comb = c->d_comb;
+    t.perm = pl.tc_perm ? c->d_perm : nullptr;
+    t.twoF = c->d_twoF;
+    t.scratch = c->d_tcs;
+    t.err = c->d_err;
+    t.n_sft = c->n_sft;
+    t.n_sky = c->n_sky;
+    t.n_fdot = c->n_fdot;
+    t.n_f = c->n_f;
+    t.n_sub = pl.tc_sub;
+    t.rps = c->n_fdot * pl.tc_sub;
+    t.rt = pl.tc_rt;
+    t.n_tiles = pl.tc_tiles;
+    t.n_colb = pl.tc_colb;
+    t.gk = pl.tc_gk;
+    t.stop = c->ring_stall;
+    return t;
+}
+
 // True when the built tables are the ones the plan's kernel reads (kind and
 // extent); the far-field and sinc kernels are never launched otherwise.
 bool tables_match(const fstat_ctx* c, const Plan& pl) {
@@ -1531,6 +1750,10 @@ bool tables_match(const fstat_ctx* c, const Plan& pl) {
 cudaError_t launch_dir(const fstat_ctx* c, const DirichletParams& dp, long long grid, cudaStream_t s) {
     const Plan& pl = c->plan;
     const int threads = pl.W * 32;
+    if (pl.tc) {
+        if (c->gt_dirty || (pl.tc_perm && c->perm_on_device != 2)) return cudaErrorInvalidValue;
+        return launch_dirichlet_tc(tc_params(c), s);
+    }
     if (pl.far) {
         if (!tables_match(c, pl)) return cudaErrorInvalidValue;
         return launch_dirichlet_far(pl.variant, dp, threads, pl.smem, grid, s);
@@ -1716,6 +1939,17 @@ int fstat_get_plan(fstat_ctx* c, int32_t* out) {
     return FSTAT_OK;
 }
 
+int fstat_get_tensor_tiles(fstat_ctx* c, int32_t* out) {
+    int32_t p[8];
+    if (!out) return FSTAT_EINVAL;
+    const int rc = fstat_get_plan(c, p);
+    if (rc != FSTAT_OK) return rc;
+    const Plan& pl = c->plan;
+    const int32_t v[4] = {pl.tc_rt, pl.tc_tiles, pl.tc_colb, pl.tc_gk}, none[4] = {0, 0, 0, 0};
+    std::memcpy(out, pl.tc ? v : none, sizeof(v));
+    return FSTAT_OK;
+}
+
 int fstat_set_noise_floor(fstat_ctx* c, int32_t half_window) {
     if (!c) return FSTAT_EINVAL;
     c->err.clear();
@@ -1812,6 +2046,38 @@ int fstat_autotune(fstat_ctx* c, void* cuda_stream, int32_t* out) {
         c->opts = saved;
         return rc;
     }
+    if (c->plan.tc) {   // nothing to tune: one tile shape; its time on a slice of about four waves
+        TcParams t = tc_params(c);
+        t.n_tiles = std::min(t.n_tiles, std::max(1, 4 * current_sm_count() / t.n_colb));
+        cudaEvent_t e0, e1;
+        cudaEventCreate(&e0);
+        cudaEventCreate(&e1);
+        float best = 1e30f;
+        cudaError_t e = launch_timing(timing_params(c, c->n_sky), s);
+        for (int rep = 0; rep < 3 && e == cudaSuccess; ++rep) {
+            cudaEventRecord(e0, s);
+            e = launch_dirichlet_tc(t, s);
+            cudaEventRecord(e1, s);
+            if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+            float ms = 0.f;
+            if (e == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
+            if (rep > 0) best = std::min(best, ms);
+        }
+        c->launches += 4;
+        cudaEventDestroy(e0);
+        cudaEventDestroy(e1);
+        if (out) {
+            out[0] = c->plan.M;
+            out[1] = c->plan.C;
+            out[2] = c->plan.W;
+            out[3] = (int32_t)std::min(best * 1000.f, 2.0e9f);
+        }
+        c->opts = saved;
+        c->plan_valid = false;
+        c->computed = false;
+        if (e != cudaSuccess) return fail(c, FSTAT_ECUDA, "autotune: %s", cudaGetErrorString(e));
+        return FSTAT_OK;
+    }
     std::vector<int> Ms;   // 0: the planner's own choice of form (the rows form where it applies)
     if (c->plan.rows) Ms = {0, 5, 7};
     else if (c->plan.two) Ms = {5, 3};
@@ -1893,6 +2159,7 @@ int fstat_batch_add(fstat_ctx* c, const fstat_workunit* wu, int32_t* wu_id) {
     int rc = fstat_create(&w, c->device, &c->opts);
     if (rc != FSTAT_OK) return fail(c, rc, "workunit context creation failed");
     w->batch_member = true;
+    w->opts0 = c->opts0;
     for (int d = 0; d < wu->n_det; ++d) {
         rc = fstat_set_sfts(w, d, &wu->det[d], wu->Tsft, wu->k_lo, wu->n_bins, wu->n_sft[d], wu->t_start[d],
                             wu->bins[d], FSTAT_MEM_HOST);
@@ -1915,7 +2182,7 @@ int fstat_batch_add(fstat_ctx* c, const fstat_workunit* wu, int32_t* wu_id) {
         w->opts.algo = FSTAT_ALGO_SINCPOLY;
         if (make_plan(w, pl) != FSTAT_OK) pl = Plan{};
     }
-    if (pl.far && (!pl.ring || pl.L != 2)) w->opts.algo = FSTAT_ALGO_DIRECT;
+    if (pl.far && !pl.tc && (!pl.ring || pl.L != 2)) w->opts.algo = FSTAT_ALGO_DIRECT;
     w->plan_valid = false;
     w->err.clear();
     c->wus.push_back(w);
@@ -1996,7 +2263,7 @@ int enqueue_batch(fstat_ctx* c, const std::vector<int>& order, const std::vector
         w->launches += 1;
     }
     CUDA_TRY(c, cudaMemcpyAsync(c->d_rem, c->d_rem_init, sizeof(int) * n, cudaMemcpyDeviceToDevice, s));
-    CUDA_TRY(c, cudaMemsetAsync(c->d_queue, 0, sizeof(unsigned long long) * groups.size(), s));
+    if (!groups.empty()) CUDA_TRY(c, cudaMemsetAsync(c->d_queue, 0, sizeof(unsigned long long) * groups.size(), s));
     const int dev_sms = current_sm_count();
     const size_t n_side = groups.empty() ? 0 : groups.size() - 1;
     while (c->side_streams.size() < n_side) {
@@ -2047,12 +2314,20 @@ int enqueue_batch(fstat_ctx* c, const std::vector<int>& order, const std::vector
         c->launches += 1;
         if (g > 0) CUDA_TRY(c, cudaEventRecord(c->side_events[g], gs));
     }
+    for (int k = 0; k < n; ++k) {   // tensor-core workunits: each fills the SMs by itself
+        fstat_ctx* w = c->wus[order[k]];
+        if (!w->plan.tc) continue;
+        cudaError_t e = launch_dir(w, DirichletParams{}, 0, s);
+        if (e != cudaSuccess) return fail(c, FSTAT_ECUDA, "batch Dirichlet launch: %s", cudaGetErrorString(e));
+        stamp_kernel<<<1, 1, 0, s>>>(c->d_done + k);
+        CUDA_TRY(c, cudaGetLastError());
+        c->launches += 2;
+    }
     for (size_t g = 1; g < groups.size(); ++g) CUDA_TRY(c, cudaStreamWaitEvent(s, c->side_events[g], 0));
     for (fstat_ctx* w : c->wus) {
         int rc = enqueue_topk(w, s);
         if (rc != FSTAT_OK) return fail(c, rc, "%s", w->err.c_str());
     }
-    (void)order;
     return FSTAT_OK;
 }
 
@@ -2072,7 +2347,7 @@ int fstat_batch_compute(fstat_ctx* c, void* cuda_stream) {
         w->stream = s;
         int rc = prepare(w, s);
         if (rc != FSTAT_OK) return fail(c, rc, "workunit: %s", w->err.c_str());
-        if (w->plan.far && (!w->plan.ring || w->plan.L != 2 || w->plan.rows || w->plan.two)) {   // persistent: direct, one-row L = 2 ring
+        if (w->plan.far && !w->plan.tc && (!w->plan.ring || w->plan.L != 2 || w->plan.rows || w->plan.two)) {   // persistent: direct, one-row L = 2 ring
             w->opts.algo = FSTAT_ALGO_DIRECT;
             w->plan_valid = false;
             c->graph_valid = false;
@@ -2090,6 +2365,7 @@ int fstat_batch_compute(fstat_ctx* c, void* cuda_stream) {
     for (int i = 0; i < n; ++i) order[i] = i;
     auto key = [&](int i) {
         const Plan& pl = c->wus[i]->plan;
+        if (pl.tc) return 1 << 21;   // after the groups of the persistent forms, one launch each
         const int resident = (int)std::min<size_t>(15, (227 * 1024) / (pl.smem + 1024));
         return (pl.ring ? 1 << 20 : 0) + pl.variant * 1024 + pl.W * 16 + resident;
     };
@@ -2102,6 +2378,7 @@ int fstat_batch_compute(fstat_ctx* c, void* cuda_stream) {
         std::vector<int> rem(n);
         for (int k = 0; k < n; ++k) {
             fstat_ctx* w = c->wus[order[k]];
+            if (w->plan.tc) continue;
             if (groups.empty() || key(order[groups.back().first]) != key(order[k])) {
                 groups.push_back(BatchGroup{w->plan.variant, w->plan.W, w->opts.bins_form, 0, k, 0, w->plan.ring});
                 prefix.push_back(0);
@@ -2120,10 +2397,10 @@ int fstat_batch_compute(fstat_ctx* c, void* cuda_stream) {
         if (c->d_queue) cudaFree(c->d_queue);
         if (c->d_done) cudaFree(c->d_done);
         CUDA_TRY(c, cudaMalloc(&c->d_banks, sizeof(DirichletParams) * n));
-        CUDA_TRY(c, cudaMalloc(&c->d_prefix, sizeof(long long) * prefix.size()));
+        CUDA_TRY(c, cudaMalloc(&c->d_prefix, sizeof(long long) * (prefix.size() + 1)));
         CUDA_TRY(c, cudaMalloc(&c->d_rem_init, sizeof(int) * n));
         CUDA_TRY(c, cudaMalloc(&c->d_rem, sizeof(int) * n));
-        CUDA_TRY(c, cudaMalloc(&c->d_queue, sizeof(unsigned long long) * groups.size()));
+        CUDA_TRY(c, cudaMalloc(&c->d_queue, sizeof(unsigned long long) * (groups.size() + 1)));
         CUDA_TRY(c, cudaMalloc(&c->d_done, sizeof(unsigned long long) * (n + 1)));
         CUDA_TRY(c, cudaMemcpy(c->d_banks, banks.data(), sizeof(DirichletParams) * n, cudaMemcpyHostToDevice));
         CUDA_TRY(c, cudaMemcpy(c->d_prefix, prefix.data(), sizeof(long long) * prefix.size(), cudaMemcpyHostToDevice));

@@ -195,6 +195,32 @@ __host__ __device__ inline RingSmem ring_smem(int stages, int w_tab, bool sinc =
     return r;
 }
 
+// Tensor-core form of the Dirichlet accumulation (dirichlet_tc.cu): tiles of
+// kTcRows rows (sky point x spindown x sub-bin offset) x kTcCols columns (one
+// bin apart).
+constexpr int kTcRows = 128, kTcCols = 64;
+constexpr int kTcBlkMax = 31;      // 4-position blocks copied for the widest window
+constexpr int kTcMaxSpread = 45;   // bins between the lowest and highest window of a tile's rows
+struct TcParams {
+    const unsigned char* gtab;     // [n_sft][n_blk][2 (high, low part)] core matrices of 128 bytes
+    const float* inv_scale;        // [n_sft] inverse of the power of two the tables are scaled by
+    int n_blk, xoff;               // 4-position blocks per SFT, position of bin k_lo
+    long long k_lo;
+    const SkySftMeta* meta;        // [n_sft][n_sky] in grouping order
+    const SkySftBase* base;        // [n_sft][n_sky]
+    const float4* comb;            // [n_sky]
+    const int* perm;               // sky point at each place of the grouping order, or null
+    float* twoF;                   // [n_sky][n_fdot][n_f]
+    float4* scratch;               // [blocks][2][kTcRows][kTcCols]
+    int* err;
+    int n_sft, n_sky, n_fdot, n_f;
+    int n_sub;                     // templates per bin: template j = n_sub * column + offset
+    int rps, rt;                   // rows per sky point, rows per tile
+    int n_tiles, n_colb;           // row tiles, column blocks
+    int gk;                        // groups of 16 positions a tile's windows span at most (2 .. 4)
+    int stop;                      // testing aid: copies stop after this many SFTs (< 0: never)
+};
+
 // Device-side description of a batch of template banks for the persistent kernel.
 struct DirichletBatch {
     const DirichletParams* banks;     // [n_wu]
@@ -279,6 +305,9 @@ cudaError_t launch_far_tables(const void* bins, int form, long long row, int n_s
 cudaError_t launch_sinc_tables(const void* bins, int form, long long row, int n_sft, int n_bins,
                                const SincGamma& gam, float4* pcoef, int n_pos, int xoff, bool split,
                                cudaStream_t s);
+cudaError_t launch_tc_tables(const void* bins, int form, long long row, int n_sft, int n_bins, int n_blk, int xoff,
+                             unsigned char* gtab, float* inv_scale, cudaStream_t s);
+cudaError_t launch_dirichlet_tc(const TcParams& p, cudaStream_t s);
 cudaError_t launch_dirichlet_far(int v, const DirichletParams& p, int threads, size_t smem, long long grid,
                                  cudaStream_t s);
 cudaError_t launch_dirichlet_far_batch(int v, const DirichletBatch& b, int threads, size_t smem, int grid,

@@ -24,9 +24,9 @@ extern "C" {
 #endif
 
 /* Largest k the call accepts; the scratch area is sized for it:
- * 3 x 2048 histogram words, 16 state words, 1024 block tie counts, one slot
- * counter and k (index, value) candidate slots = 225,348 bytes, rounded up to
- * 225,536 (a multiple of 256). */
+ * 16 state words, 4 x 2048 histogram words, 32768 group maxima, 1024 block tie
+ * counts and 20480 (index, value) candidate slots = 413,760 bytes, rounded up
+ * to 413,952 (a multiple of 256). */
 #define FSTAT_NOALLOC_MAX_K 16384
 
 /* The k largest values of v[0 .. n-1] (device FP32, n >= 1, values >= 0 and
@@ -43,8 +43,8 @@ extern "C" {
  * Everything runs asynchronously on cuda_stream (NULL = the legacy default
  * stream) on `device`, which becomes the calling thread's current device.
  *
- * Scratch: a static device array of the size above.  Its histogram, state and
- * slot-counter words must start at zero for each call; the call clears them
+ * Scratch: a static device array of the size above.  Its histogram and
+ * state words must start at zero for each call; the call clears them
  * itself with cudaMemsetAsync on cuda_stream before its first kernel, so the
  * caller has nothing to prepare and may rely on nothing it leaves behind.
  * Because there is one scratch area per device, calls on the same device whose

@@ -1110,22 +1110,11 @@ int ensure_topk(fstat_ctx* c) {
     if (k <= 0) return FSTAT_OK;
     if (c->tw_k >= k) return FSTAT_OK;
     TopkWork& w = c->tw;
-    cudaFree(w.hist);
-    cudaFree(w.state);
-    cudaFree(w.tie_count);
-    cudaFree(w.cand_idx);
-    cudaFree(w.cand_val);
-    cudaFree(w.n_cand);
+    cudaFree(w.scratch);
     cudaFree(w.out_idx);
     cudaFree(w.out_val);
     w = TopkWork{};
-    w.n_blocks = 1024;
-    CUDA_TRY(c, cudaMalloc(&w.hist, sizeof(unsigned int) * 3 * 2048));
-    CUDA_TRY(c, cudaMalloc(&w.state, sizeof(unsigned int) * 16));
-    CUDA_TRY(c, cudaMalloc(&w.tie_count, sizeof(unsigned int) * w.n_blocks));
-    CUDA_TRY(c, cudaMalloc(&w.cand_idx, sizeof(long long) * k));
-    CUDA_TRY(c, cudaMalloc(&w.cand_val, sizeof(float) * k));
-    CUDA_TRY(c, cudaMalloc(&w.n_cand, sizeof(unsigned int)));
+    CUDA_TRY(c, cudaMalloc(&w.scratch, kTopkScratch));
     CUDA_TRY(c, cudaMalloc(&w.out_idx, sizeof(long long) * k));
     CUDA_TRY(c, cudaMalloc(&w.out_val, sizeof(float) * k));
     c->tw_k = k;
@@ -1260,8 +1249,7 @@ void fstat_destroy(fstat_ctx* c) {
     if (c->bev1) cudaEventDestroy(c->bev1);
     void* ptrs[] = {c->d_fstart, c->d_base, c->d_bins, c->d_bins16, c->d_scale, c->d_state, c->d_tstart, c->d_det_of, c->d_sky,
                     c->d_fdot, c->d_meta, c->d_kh0, c->d_ph0, c->d_abcd, c->d_comb, c->d_twoF, c->d_err,
-                    c->tw.hist, c->tw.state, c->tw.tie_count, c->tw.cand_idx, c->tw.cand_val, c->tw.n_cand,
-                    c->tw.out_idx, c->tw.out_val, c->d_inj_work, c->d_sig, c->d_ptab, c->d_pcoef,
+                    c->tw.scratch, c->tw.out_idx, c->tw.out_val, c->d_inj_work, c->d_sig, c->d_ptab, c->d_pcoef,
                     c->d_bins_w, c->d_floor, c->d_sbar, c->d_weight, c->d_cov, c->d_comb_j, c->d_slide_seg, c->d_slide_A,
                     c->d_slide_B, c->d_slide_out, c->d_perm, c->d_rank, c->d_gtab, c->d_inv, c->d_tcs};
     for (void* p : ptrs)
@@ -1770,7 +1758,7 @@ int enqueue_topk(fstat_ctx* c, cudaStream_t s) {
     const int k = (int)std::min<long long>(c->opts.topk, n);
     if (k > 0) {
         CUDA_TRY(c, launch_topk(c->d_twoF, n, k, c->tw, s));
-        c->launches += 9;   // 3 histograms, 3 selections, collect, ties, sort
+        c->launches += topk_launches(n, k);
     }
     return FSTAT_OK;
 }

@@ -287,17 +287,12 @@ cudaError_t launch_patches(const float* twoF, int n_f, int n_d, int s_a, int s_d
 cudaError_t launch_windows(const float* twoF, int n_f, int n_a, int n_d, int s_a, int s_d, int n_fp,
                            const int* origin_dev, int n_w, float shift, float scale, void* out, cudaStream_t s);
 
-// Toplist (radix select over the FP32 bit patterns of 2F >= 0).
+// Toplist of the K <= 16384 largest 2F >= 0.
+constexpr size_t kTopkScratch = 413952;   // bytes, whatever the bank and K
 struct TopkWork {
-    unsigned int* hist;        // [3][2048]
-    unsigned int* state;       // [16] prefix, threshold, counts
-    unsigned int* tie_count;   // [n_blocks]
-    long long* cand_idx;       // [topk]
-    float* cand_val;           // [topk]
-    unsigned int* n_cand;      // [1]
+    unsigned int* scratch;     // kTopkScratch bytes, 256-byte aligned
     long long* out_idx;        // [topk]
     float* out_val;            // [topk]
-    int n_blocks;
 };
 cudaError_t launch_far_tables(const void* bins, int form, long long row, int n_sft, int n_bins, const FarGamma& gam,
                               float4* ptab, float4* pcoef, int n_pos, int xoff, cudaStream_t s);
@@ -313,6 +308,7 @@ cudaError_t launch_dirichlet_far(int v, const DirichletParams& p, int threads, s
 cudaError_t launch_dirichlet_far_batch(int v, const DirichletBatch& b, int threads, size_t smem, int grid,
                                        cudaStream_t s);
 cudaError_t dirichlet_far_batch_occupancy(int v, int threads, size_t smem, int* blocks_per_sm);
+int topk_launches(long long n, int k);   // kernels that launch_topk launches
 cudaError_t launch_topk(const float* v, long long n, int k, TopkWork& w, cudaStream_t s);
 
 // One segment of a stack-slide: its device 2F [n_sky][n_fdot][n_f] and grid.

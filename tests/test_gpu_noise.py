@@ -78,3 +78,23 @@ def test_noise_floor_errors(lib):
         assert e.value.code == lib.FSTAT_ESTATE
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("half,n_bins", [(1, 200), (15, 200), (16, 200), (31, 201), (32, 200), (47, 263), (48, 200),
+                                         (63, 200), (64, 257), (64, 100)])
+def test_floor_is_exact_at_every_window_width(lib, half, n_bins):
+    """Windows that fill 1 to 5 values a lane, wider than the band too; small
+    whole-number bins, so that most powers are equal to others and some are 0."""
+    w = config_mid(seed=half, n_sft=9, n_sky=1, n_f=10, n_fdot=1, n_bins=n_bins)
+    rng = np.random.default_rng(half)
+    bins = [(rng.integers(-2, 3, (d.n_sft, w.n_bins)) + 1j * rng.integers(-2, 3, (d.n_sft, w.n_bins))).astype(np.complex64)
+            for d in w.detectors]
+    g = lib.FStat(0, dterms=w.dterms, topk=5)
+    try:
+        g.load_workload(w, bins_override=bins)
+        lib.fstat_set_noise_floor(g.ctx, half)
+        g.compute()
+        fl, _ = lib.fstat_get_noise(g.ctx, w.n_sft_total, w.n_bins)
+    finally:
+        g.close()
+    np.testing.assert_array_equal(fl, np.concatenate([N.running_median_floor(b, half) for b in bins]))

@@ -65,46 +65,47 @@ __global__ void sft_state_kernel(const double* __restrict__ t_start, const int* 
     out[i] = s;
 }
 
-struct SkyFrame {
-    double n[3], X[3], Y[3];
+// What a sky point contributes: the unit vector to it over c, and the
+// coefficients of a = X.D.X - Y.D.Y and b = 2 X.D.Y in the six components of
+// the detector tensor D, with X, Y the polarisation axes at the point.  A
+// (sky point, SFT) pair then takes 6 products for each pair of results
+// instead of the 35 operations and 2 divisions of forming D.X and D.Y.
+struct SkyCoef {
+    double nc[3], qa[6], qb[6];
 };
 
-__device__ __forceinline__ SkyFrame sky_frame(double alpha, double delta) {
+__device__ __forceinline__ SkyCoef sky_coef(double alpha, double delta) {
     double sa, ca, sd, cd;
     sincos(alpha, &sa, &ca);
     sincos(delta, &sd, &cd);
-    SkyFrame f;
-    f.n[0] = cd * ca;
-    f.n[1] = cd * sa;
-    f.n[2] = sd;
-    f.X[0] = -sa;
-    f.X[1] = ca;
-    f.X[2] = 0.0;
-    f.Y[0] = -sd * ca;
-    f.Y[1] = -sd * sa;
-    f.Y[2] = cd;
+    const double X[3] = {-sa, ca, 0.0}, Y[3] = {-sd * ca, -sd * sa, cd};
+    SkyCoef f;
+    f.nc[0] = cd * ca / kC;
+    f.nc[1] = cd * sa / kC;
+    f.nc[2] = sd / kC;
+    int k = 0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = i; j < 3; ++j, ++k) {
+            f.qa[k] = (i == j ? 1.0 : 2.0) * (X[i] * X[j] - Y[i] * Y[j]);
+            f.qb[k] = i == j ? 2.0 * X[i] * Y[i] : 2.0 * (X[i] * Y[j] + X[j] * Y[i]);
+        }
     return f;
 }
 
-// dtau, tdot, a, b of one SFT for one sky frame.
-__device__ __forceinline__ void timing_antenna(const SftState& s, const SkyFrame& f, double t_ref,
+// dtau, tdot, a, b of one SFT for one sky point.
+__device__ __forceinline__ void timing_antenna(const SftState& s, const SkyCoef& f, double t_ref,
                                                double& dtau, double& tdot, double& a, double& b) {
-    const double nr = f.n[0] * s.r[0] + f.n[1] * s.r[1] + f.n[2] * s.r[2];
-    const double nv = f.n[0] * s.v[0] + f.n[1] * s.v[1] + f.n[2] * s.v[2];
-    dtau = (s.t_mid - t_ref) + nr / kC;
-    tdot = 1.0 + nv / kC;
-    const double* D = s.dt;
-    const double DX[3] = {D[0] * f.X[0] + D[1] * f.X[1] + D[2] * f.X[2],
-                          D[1] * f.X[0] + D[3] * f.X[1] + D[4] * f.X[2],
-                          D[2] * f.X[0] + D[4] * f.X[1] + D[5] * f.X[2]};
-    const double DY[3] = {D[0] * f.Y[0] + D[1] * f.Y[1] + D[2] * f.Y[2],
-                          D[1] * f.Y[0] + D[3] * f.Y[1] + D[4] * f.Y[2],
-                          D[2] * f.Y[0] + D[4] * f.Y[1] + D[5] * f.Y[2]};
-    const double xdx = f.X[0] * DX[0] + f.X[1] * DX[1] + f.X[2] * DX[2];
-    const double ydy = f.Y[0] * DY[0] + f.Y[1] * DY[1] + f.Y[2] * DY[2];
-    const double xdy = f.X[0] * DY[0] + f.X[1] * DY[1] + f.X[2] * DY[2];
-    a = xdx - ydy;
-    b = 2.0 * xdy;
+    dtau = (s.t_mid - t_ref) + (f.nc[0] * s.r[0] + f.nc[1] * s.r[1] + f.nc[2] * s.r[2]);
+    tdot = 1.0 + (f.nc[0] * s.v[0] + f.nc[1] * s.v[1] + f.nc[2] * s.v[2]);
+    a = f.qa[0] * s.dt[0];
+    b = f.qb[0] * s.dt[0];
+#pragma unroll
+    for (int k = 1; k < 6; ++k) {
+        a = fma(f.qa[k], s.dt[k], a);
+        b = fma(f.qb[k], s.dt[k], b);
+    }
 }
 
 constexpr double kTwo32 = 4294967296.0;
@@ -116,12 +117,8 @@ __device__ __forceinline__ unsigned int frac_fx32(double x) {
     return (unsigned int)(unsigned long long)(long long)s;   // 2^32 wraps to 0
 }
 
-// Absolute bin position as 32.32 fixed point.
-__device__ __forceinline__ long long bin_fx(double khat) {
-    const double hi = floor(khat);
-    const double lo = rint((khat - hi) * kTwo32);
-    return ((long long)hi << 32) + (long long)lo;
-}
+// x bins as 32.32 fixed point, from x 2^32 (the scaling is exact).
+__device__ __forceinline__ long long bin_fx(double x_two32) { return llrint(x_two32); }
 
 template <int BLOCK>
 __device__ __forceinline__ double block_sum(double v, double* red) {
@@ -140,11 +137,23 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 
 constexpr int kTimingBlock = 256;
 
+// Bound: the FP64 pipe (2 lanes a clock and SM), about 50 operations a pair; so
+// the sky point's coefficients are formed by one warp, constants are folded, and
+// the spindown steps are left out where there is one spindown.  2048 sky points
+// x 1600 SFTs: 420 us against 742 us with the frames in every thread, two
+// divisions and 105 operations a pair.
 __global__ void __launch_bounds__(kTimingBlock) timing_kernel(const TimingParams p) {
     __shared__ double red[3][kTimingBlock / 32];
+    __shared__ SkyCoef coef;
     const int sky = blockIdx.x;
-    const SkyFrame fr = sky_frame(p.sky[2 * sky], p.sky[2 * sky + 1]);
+    if (threadIdx.x < 32) {
+        const SkyCoef f = sky_coef(p.sky[2 * sky], p.sky[2 * sky + 1]);
+        if (threadIdx.x == 0) coef = f;
+    }
+    __syncthreads();
+    const SkyCoef fr = coef;
     const double kconst = 2.0 / kPi;   // pair form of the Dirichlet sum and the 1/pi of sin(pi kappa)/pi
+    const double bins32 = p.T * kTwo32, df32 = p.df * bins32;
     double sAA = 0.0, sBB = 0.0, sAB = 0.0;
     for (int i = threadIdx.x; i < p.n_sft; i += kTimingBlock) {
         const SftState s = p.st[i];
@@ -158,15 +167,14 @@ __global__ void __launch_bounds__(kTimingBlock) timing_kernel(const TimingParams
         sAA += a * a;
         sBB += b * b;
         sAB += a * b;
-        const double dk_real = p.df * tdot * p.T;
-        const long long dk = llrint(dk_real * kTwo32);
+        const long long dk = llrint(df32 * tdot);
         const long long pdk = (long long)p.P * dk;
         SkySftMeta m;
         m.dk = dk;
         m.span = (long long)(p.M - 1) * pdk;
         const unsigned int dphi = frac_fx32(p.df * dtau);
         m.dphi = dphi;
-        m.eps = (float)((double)(pdk - ((long long)p.L << 32)) / kTwo32);
+        m.eps = (float)(pdk - ((long long)p.L << 32)) * 2.3283064365386963e-10f;   // x 2^-32
         // twiddle step e^{-2 pi i (P dphi + L/2)} from the same fixed-point step:
         // a reduced angle (the step in [-1/2, 1/2) cycle) whose sine and cosine
         // are stored in FP32, so they are taken in FP32 (error ~2e-7 rad from
@@ -184,10 +192,16 @@ __global__ void __launch_bounds__(kTimingBlock) timing_kernel(const TimingParams
         if (p.uniform) {
             const double fd = p.fdot[0];
             SkySftBase bs;
-            bs.kh0 = bin_fx((p.f0 + fd * dtau) * tdot * p.T);
-            bs.dkh = llrint(p.dfdot * dtau * tdot * p.T * kTwo32);
+            const double tb = tdot * bins32;
+            bs.kh0 = bin_fx((p.f0 + fd * dtau) * tb);
             bs.ph0 = frac_fx32(p.f0 * dtau + 0.5 * fd * dtau * dtau);
-            bs.dph = frac_fx32(0.5 * p.dfdot * dtau * dtau);
+            bs.dkh = 0;
+            bs.dph = 0u;
+            if (p.dfdot != 0.0) {
+                const double dd = p.dfdot * dtau;
+                bs.dkh = llrint(dd * tb);
+                bs.dph = frac_fx32(0.5 * dd * dtau);
+            }
             // twiddle step from one spindown row to the next, e^{-2 pi i dph}
             // (read by the row-tiled forms only)
             float rs = 0.f, rc = 1.f;
@@ -201,7 +215,7 @@ __global__ void __launch_bounds__(kTimingBlock) timing_kernel(const TimingParams
         } else {
             for (int d = 0; d < p.n_fdot; ++d) {
                 const double fd = p.fdot[d];
-                const double khat0 = (p.f0 + fd * dtau) * tdot * p.T;
+                const double khat0 = (p.f0 + fd * dtau) * (tdot * bins32);
                 const double cyc0 = p.f0 * dtau + 0.5 * fd * dtau * dtau;
                 const size_t o = ((size_t)sky * p.n_fdot + d) * p.n_sft + i;
                 const long long kfx = bin_fx(khat0);
@@ -248,7 +262,7 @@ __global__ void __launch_bounds__(kTimingBlock) coverage_comb_kernel(const Timin
     const int n1 = n_f + 1;
     for (int t = threadIdx.x; t < 3 * n1; t += kTimingBlock) cdiff[t] = 0ull;
     __syncthreads();
-    const SkyFrame fr = sky_frame(p.sky[2 * sky], p.sky[2 * sky + 1]);
+    const SkyCoef fr = sky_coef(p.sky[2 * sky], p.sky[2 * sky + 1]);
     for (int i = threadIdx.x; i < p.n_sft; i += kTimingBlock) {
         const int2 c = cov[i];
         const int lo = max(0, min(c.x, n_f)), hi = max(0, min(c.y, n_f));
@@ -316,7 +330,7 @@ __global__ void sft_timing_one_kernel(const SftState* __restrict__ st, int n_sft
                                       double delta, double t_ref, double* __restrict__ out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_sft) return;
-    const SkyFrame fr = sky_frame(alpha, delta);
+    const SkyCoef fr = sky_coef(alpha, delta);
     double dtau, tdot, a, b;
     timing_antenna(st[i], fr, t_ref, dtau, tdot, a, b);
     out[i] = dtau;
@@ -339,7 +353,7 @@ __global__ void __launch_bounds__(kTimingBlock) inject_prep_kernel(const SftStat
     __shared__ double sh_h0;
     const fstat_signal g = sig[blockIdx.x];
     double* w = work + (size_t)blockIdx.x * (kInjHead + 4 * (size_t)n_sft);
-    const SkyFrame fr = sky_frame(g.alpha, g.delta);
+    const SkyCoef fr = sky_coef(g.alpha, g.delta);
     // unit-amplitude complex amplitudes: h = Re[(a ca + b cb) e^{i Phi}]
     const double ap = (1.0 + g.cosi * g.cosi) / 2.0, ax = g.cosi;
     double s2p, c2p, sp0, cp0;

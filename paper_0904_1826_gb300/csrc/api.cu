@@ -1095,9 +1095,14 @@ bool all_finite(const double* v, size_t n) {
     return true;
 }
 
-__global__ void finite_check_kernel(const float* v, long long n, int* bad) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        if (!isfinite(v[i])) atomicOr(bad, 1);
+// v is 16-byte aligned, n a multiple of 4 (whole rows of the store)
+__global__ void finite_check_kernel(const float4* v, long long n4, int* bad) {
+    bool ok = true;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n4; i += (long long)gridDim.x * blockDim.x) {
+        const float4 x = v[i];
+        ok = ok && isfinite(x.x) && isfinite(x.y) && isfinite(x.z) && isfinite(x.w);
+    }
+    if (!ok) atomicOr(bad, 1);
 }
 
 __global__ void fill_kernel(float* v, long long n, float x) {
@@ -1390,14 +1395,6 @@ int fstat_set_sfts(fstat_ctx* c, int32_t det_index, const fstat_detector* det, d
         else if (c->det[d].set) total += (int)c->det[d].t_start.size();
     }
     if (total > 65535) return fail(c, FSTAT_EINVAL, "more than 65535 SFTs in one context");
-    // host staging for device input: validate values
-    std::vector<float> hb;
-    const float* src = bins;
-    const size_t n_el = (size_t)n_sft * n_bins * 2;
-    if (mem == FSTAT_MEM_HOST) {
-        for (size_t i = 0; i < n_el; ++i)
-            if (!std::isfinite(bins[i])) return fail(c, FSTAT_EINVAL, "non-finite SFT bin at %zu", i);
-    }
     // new device store; copy kept detectors over
     float2* nb = nullptr;
     CUDA_TRY(c, cudaMalloc(&nb, (size_t)total * row * sizeof(float2)));
@@ -1411,25 +1408,29 @@ int fstat_set_sfts(fstat_ctx* c, int32_t det_index, const fstat_detector* det, d
         }
         old_first += n_old;
     }
-    CUDA_TRY(c, cudaMemcpy2DAsync(nb + (size_t)first_of[det_index] * row, row * sizeof(float2), src,
+    CUDA_TRY(c, cudaMemcpy2DAsync(nb + (size_t)first_of[det_index] * row, row * sizeof(float2), bins,
                                   (size_t)n_bins * sizeof(float2), (size_t)n_bins * sizeof(float2), n_sft,
                                   mem == FSTAT_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
                                   c->stream));
-    if (mem == FSTAT_MEM_DEVICE) {
-        int* bad = c->d_err + 3;
-        CUDA_TRY(c, cudaMemsetAsync(bad, 0, sizeof(int), c->stream));
-        finite_check_kernel<<<256, 256, 0, c->stream>>>(bins, (long long)n_el, bad);
-        CUDA_TRY(c, cudaGetLastError());
-        c->launches += 1;
-        int hbad = 0;
-        CUDA_TRY(c, cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-        CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-        if (hbad) {
-            cudaFree(nb);
-            return fail(c, FSTAT_EINVAL, "non-finite SFT bin in device input");
-        }
-    }
+    // the copied rows (padding is zero) are checked on the device: 35 MB in 10 us, a
+    // host loop over them took 3 ms.  Nothing of the context has changed yet.
+    int* bad = c->d_err + 3;
+    int hbad = 0;
+    CUDA_TRY(c, cudaMemsetAsync(bad, 0, sizeof(int), c->stream));
+    finite_check_kernel<<<4 * current_sm_count(), 256, 0, c->stream>>>(
+        reinterpret_cast<const float4*>(nb + (size_t)first_of[det_index] * row), (long long)n_sft * row / 2, bad);
+    CUDA_TRY(c, cudaGetLastError());
+    c->launches += 1;
+    CUDA_TRY(c, cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+    if (hbad) {
+        cudaFree(nb);
+        if (mem == FSTAT_MEM_DEVICE) return fail(c, FSTAT_EINVAL, "non-finite SFT bin in device input");
+        const size_t n_el = (size_t)n_sft * n_bins * 2;
+        size_t i = 0;
+        while (i < n_el && std::isfinite(bins[i])) ++i;
+        return fail(c, FSTAT_EINVAL, "non-finite SFT bin at %zu", i);
+    }
     if (c->d_bins) cudaFree(c->d_bins);
     c->d_bins = nb;
     c->row = row;

@@ -412,27 +412,63 @@ SincGamma sinc_gamma() {
     return G;
 }
 
-// Bound, in bins, on how far apart the windows of a tile's rows can start
-// (tensor-core form): rows are (sky place, spindown, sub-bin offset) in
-// grouping order, rt rows a tile.  Two sky points' khat differ by at most
-// f_max T 1.1e-4 |n_1 - n_2| and |n_1 - n_2| <= 2 max |n - mean n| over the
-// tile; the spindowns spread it by |fdot range| tau T, the offsets by less
+// Sky points for the tensor-core form's tiles: ecliptic x, y and the unit vector.
+// The orbital velocity lies in the ecliptic plane, so what a tile's points differ
+// by in it decides how far apart their windows start; their ecliptic z hardly
+// counts (Earth's rotation only).
+struct TcSky {
+    double x, y, u[3];
+};
+std::vector<TcSky> tc_sky(const fstat_ctx* c) {
+    const double ce = std::cos(kObliquity), se = std::sin(kObliquity);
+    std::vector<TcSky> v(c->n_sky);
+    for (int i = 0; i < c->n_sky; ++i) {
+        const double al = c->h_sky[2 * i], de = c->h_sky[2 * i + 1];
+        double* u = v[i].u;
+        u[0] = std::cos(de) * std::cos(al);
+        u[1] = std::cos(de) * std::sin(al);
+        u[2] = std::sin(de);
+        v[i].x = u[0];
+        v[i].y = ce * u[1] + se * u[2];
+    }
+    return v;
+}
+
+// Bound, in bins, on how far apart the windows of a tile's rows can start; rows
+// are (sky place, spindown, sub-bin offset) in grouping order, rt rows a tile.
+// khat = (f0 + fd dtau + j df) T (1 + n.v / c): two sky points differ by at most
+// f_max T times 9.94e-5 (orbit) their distance along the velocity, here along the
+// worst of all directions in the ecliptic plane (16 are tried; 1.005 covers those
+// between), and 1.56e-6 (rotation) their whole distance; the spindowns spread it
+// by |fdot range| tau T and the points' light-travel times; the offsets by less
 // than a bin.
-double tc_spread_bins(const fstat_ctx* c, const std::vector<double>& unit, int rps, int rt, const std::vector<int>* order) {
-    const double k_max = (c->f0 + (c->n_f - 1) * c->df) * c->T;
-    double r_max = 0.0;
+double tc_spread_bins(const fstat_ctx* c, const std::vector<TcSky>& sky, int rps, int rt, const std::vector<int>* order) {
+    constexpr int kDir = 16;
+    double dx[kDir], dy[kDir];
+    for (int i = 0; i < kDir; ++i) {
+        dx[i] = std::cos(kPi * i / kDir);
+        dy[i] = std::sin(kPi * i / kDir);
+    }
+    double worst = 0.0;
     const long long n_rows = (long long)c->n_sky * rps;
     for (long long g0 = 0; g0 < n_rows; g0 += rt) {
         const int a = (int)(g0 / rps), b = (int)((std::min(n_rows, g0 + rt) - 1) / rps);
-        double m[3] = {0, 0, 0};
-        for (int i = a; i <= b; ++i)
-            for (int k = 0; k < 3; ++k) m[k] += unit[3 * (order ? (*order)[i] : i) + k];
-        for (int k = 0; k < 3; ++k) m[k] /= b - a + 1;
+        double lo[kDir], hi[kDir], m[3] = {0, 0, 0}, r2 = 0.0, width = 0.0;
         for (int i = a; i <= b; ++i) {
-            const double* u = &unit[3 * (order ? (*order)[i] : i)];
-            const double q = (u[0] - m[0]) * (u[0] - m[0]) + (u[1] - m[1]) * (u[1] - m[1]) + (u[2] - m[2]) * (u[2] - m[2]);
-            r_max = std::max(r_max, q);
+            const TcSky& p = sky[order ? (*order)[i] : i];
+            for (int k = 0; k < 3; ++k) m[k] += p.u[k] / (b - a + 1);
+            for (int k = 0; k < kDir; ++k) {
+                const double q = p.x * dx[k] + p.y * dy[k];
+                lo[k] = i == a ? q : std::min(lo[k], q);
+                hi[k] = i == a ? q : std::max(hi[k], q);
+            }
         }
+        for (int i = a; i <= b; ++i) {
+            const double* u = sky[order ? (*order)[i] : i].u;
+            r2 = std::max(r2, (u[0] - m[0]) * (u[0] - m[0]) + (u[1] - m[1]) * (u[1] - m[1]) + (u[2] - m[2]) * (u[2] - m[2]));
+        }
+        for (int k = 0; k < kDir; ++k) width = std::max(width, hi[k] - lo[k]);
+        worst = std::max(worst, 9.94e-5 * 1.005 * width + 1.56e-6 * 2.0 * std::sqrt(r2));
     }
     double fd_min = c->h_fdot[0], fd_max = c->h_fdot[0], tau = 0.0;
     for (double v : c->h_fdot) {
@@ -441,45 +477,39 @@ double tc_spread_bins(const fstat_ctx* c, const std::vector<double>& unit, int r
     }
     for (int d = 0; d < kMaxDet; ++d)
         for (double t : c->det[d].t_start) tau = std::max(tau, std::fabs(t + 0.5 * c->T - c->t_ref));
-    return k_max * 1.1e-4 * 2.0 * std::sqrt(r_max) + (fd_max - fd_min) * (tau + 500.0) * c->T * 1.00011 + 2.0;
+    const double k_max = (c->f0 + (c->n_f - 1) * c->df + std::max(std::fabs(fd_min), std::fabs(fd_max)) * (tau + 510.0)) * c->T;
+    return k_max * worst + ((fd_max - fd_min) * (tau + 510.0) + std::max(std::fabs(fd_min), std::fabs(fd_max)) * 1020.0) *
+                               c->T * 1.00011 + 2.0;
 }
 
-// Sky points in bands of delta, alpha back and forth, for tiles of g
-// consecutive points (a square patch of g of n points is side = sqrt(4 pi g /
-// n) wide).  by_count = false: bands of equal width in delta, about `side`.
-// true: from the south pole up, each band takes the points of as many whole
-// tiles as its circumference has sides, which follows the density of the list
-// and leaves no tile across two bands.  Largest distance of a point from its
-// tile's mean, lattice skies, tiles of 128 rows (equal width / by count):
-// 3001 points of one spindown 1.09 / 0.58, 20 000 0.43 / 0.23, 4000 of ten
-// 0.28 / 0.22, 1500 of seven 0.45 / 0.57.
-std::vector<int> tc_neighbour_order(const fstat_ctx* c, double g, bool by_count) {
-    const int n = c->n_sky;
-    const double side = std::sqrt(4.0 * kPi * std::max(1.0, g) / n);
-    std::vector<double> alpha(n);
-    for (int i = 0; i < n; ++i) {
-        alpha[i] = std::fmod(c->h_sky[2 * i], 2.0 * kPi);
-        if (alpha[i] < 0) alpha[i] += 2.0 * kPi;
-    }
+// Sky points in strips of ecliptic x, y back and forth, for tiles of g
+// consecutive points: a strip takes points until its tiles are as long as it is
+// wide, and whole tiles, so that none lies across two strips.  Both hemispheres
+// fall on the same x, y, which halves a tile's extent there against patches of
+// the sphere: spread of 128-row tiles, lattice skies, bins (patches of equal
+// right ascension and declination / this order): 250 points x 7 spindowns at 217
+// Hz 80 / 37; 4000 x 10 at 100 Hz 10 / 6; 3001 x 1 at 120 Hz 30 / 18.
+std::vector<int> tc_neighbour_order(const std::vector<TcSky>& sky, double g) {
+    const int n = (int)sky.size();
     std::vector<int> order(n);
     for (int i = 0; i < n; ++i) order[i] = i;
-    auto delta = [&](int i) { return c->h_sky[2 * (size_t)i + 1]; };
-    std::sort(order.begin(), order.end(), [&](int x, int y) { return delta(x) < delta(y) || (delta(x) == delta(y) && x < y); });
-    const double width = kPi / std::max(1.0, std::round(kPi / side));
+    std::sort(order.begin(), order.end(),
+              [&](int a, int b) { return sky[a].x < sky[b].x || (sky[a].x == sky[b].x && a < b); });
     bool back = false;
     for (int i = 0; i < n; back = !back) {
+        double lo = sky[order[i]].y, hi = lo;
         int m = 0;
-        if (by_count) {
-            const double mid = std::min(delta(order[i]) + 0.5 * side, 0.5 * kPi);
-            m = (int)std::min<double>(n - i, std::round(g * std::max(1.0, std::round(2.0 * kPi * std::cos(mid) / side))));
-            if (m < 1 || n - i - m < 0.5 * g) m = n - i;
-        } else {
-            const double b = std::floor((delta(order[i]) + 0.5 * kPi) / width);
-            while (i + m < n && (m == 0 || std::floor((delta(order[i + m]) + 0.5 * kPi) / width) == b)) ++m;
+        while (i + m < n) {
+            const TcSky& p = sky[order[i + m++]];
+            lo = std::min(lo, p.y);
+            hi = std::max(hi, p.y);
+            if (m >= g && m * (p.x - sky[order[i]].x) >= g * (hi - lo)) break;
         }
-        std::sort(order.begin() + i, order.begin() + i + m, [&](int x, int y) {
-            if (alpha[x] != alpha[y]) return back ? alpha[x] > alpha[y] : alpha[x] < alpha[y];
-            return x < y;
+        m = (int)std::min<double>(n - i, std::max(1.0, std::round(std::max(1.0, std::round(m / g)) * g)));
+        if (n - i - m < 0.5 * g) m = n - i;
+        std::sort(order.begin() + i, order.begin() + i + m, [&](int a, int b) {
+            if (sky[a].y != sky[b].y) return back ? sky[a].y > sky[b].y : sky[a].y < sky[b].y;
+            return a < b;
         });
         i += m;
     }
@@ -513,25 +543,16 @@ void choose_tc(fstat_ctx* c, int P, int L, bool found, Plan& pl) {
     const double t_other = (double)c->n_sky * c->n_fdot * c->n_f * c->n_sft / rate;
     if (n_rows > (1 << 28) || (n_rows / 32 + 1) * colb > (1 << 28) || t_other > 3000.0) return;   // 32-bit counters
     if (t_tc(kTcRows) > 0.92 * t_other) return;
-    std::vector<double> unit(3 * (size_t)c->n_sky);
-    for (int i = 0; i < c->n_sky; ++i) {
-        const double al = c->h_sky[2 * i], de = c->h_sky[2 * i + 1];
-        unit[3 * i] = std::cos(de) * std::cos(al);
-        unit[3 * i + 1] = std::cos(de) * std::sin(al);
-        unit[3 * i + 2] = std::sin(de);
-    }
+    const std::vector<TcSky> sky = tc_sky(c);
     for (int rt = kTcRows; rt >= 32 && t_tc(rt) <= 0.92 * t_other; rt /= 2) {
-        double spread = tc_spread_bins(c, unit, rps, rt, nullptr);
-        bool nat = true;
+        double spread = tc_spread_bins(c, sky, rps, rt, nullptr);
         c->perm_on_device = 0;
-        for (const bool by_count : {false, true}) {
-            std::vector<int> order = tc_neighbour_order(c, (double)rt / rps, by_count);
-            const double q = tc_spread_bins(c, unit, rps, rt, &order);
-            if (q < spread) {
-                spread = q;
-                nat = false;
-                c->tc_order = std::move(order);
-            }
+        std::vector<int> order = tc_neighbour_order(sky, (double)rt / rps);
+        const double q = tc_spread_bins(c, sky, rps, rt, &order);
+        const bool nat = spread <= q;
+        if (!nat) {
+            spread = q;
+            c->tc_order = std::move(order);
         }
         if (spread > kTcMaxSpread) continue;
         pl.tc = true;

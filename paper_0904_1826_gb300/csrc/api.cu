@@ -483,13 +483,13 @@ double tc_spread_bins(const fstat_ctx* c, const std::vector<TcSky>& sky, int rps
 }
 
 // Sky points in strips of ecliptic x, y back and forth, for tiles of g
-// consecutive points: a strip takes points until its tiles are as long as it is
-// wide, and whole tiles, so that none lies across two strips.  Both hemispheres
+// consecutive points: a strip takes points until its tiles are `length` times as
+// long as it is wide, and whole tiles, so that none lies across two strips.  Both hemispheres
 // fall on the same x, y, which halves a tile's extent there against patches of
 // the sphere: spread of 128-row tiles, lattice skies, bins (patches of equal
 // right ascension and declination / this order): 250 points x 7 spindowns at 217
 // Hz 80 / 37; 4000 x 10 at 100 Hz 10 / 6; 3001 x 1 at 120 Hz 30 / 18.
-std::vector<int> tc_neighbour_order(const std::vector<TcSky>& sky, double g) {
+std::vector<int> tc_neighbour_order(const std::vector<TcSky>& sky, double g, double length) {
     const int n = (int)sky.size();
     std::vector<int> order(n);
     for (int i = 0; i < n; ++i) order[i] = i;
@@ -503,7 +503,7 @@ std::vector<int> tc_neighbour_order(const std::vector<TcSky>& sky, double g) {
             const TcSky& p = sky[order[i + m++]];
             lo = std::min(lo, p.y);
             hi = std::max(hi, p.y);
-            if (m >= g && m * (p.x - sky[order[i]].x) >= g * (hi - lo)) break;
+            if (m >= g && length * m * (p.x - sky[order[i]].x) >= g * (hi - lo)) break;
         }
         m = (int)std::min<double>(n - i, std::max(1.0, std::round(std::max(1.0, std::round(m / g)) * g)));
         if (n - i - m < 0.5 * g) m = n - i;
@@ -532,12 +532,13 @@ void choose_tc(fstat_ctx* c, int P, int L, bool found, Plan& pl) {
     const long long colb = (n_col + kTcCols - 1) / kTcCols;
     const int sms = current_sm_count();
     // Measured on GB300: a block takes 1.44 us an SFT for a tile of 128 x 64
-    // templates, whatever part of it is filled; the other forms 5.6e11 pairs/s on
+    // templates, whatever part of it is filled, and the blocks share the steps evenly; the
+    // other forms 5.6e11 pairs/s on
     // large banks of three or more spindowns, 4.6e11 on one or two, and 2.7e11
     // where the steps are 1/8 bin (L = 1); smaller banks leave them slower.
     auto t_tc = [&](int rt) {
         const long long items = ((n_rows + rt - 1) / rt) * colb;
-        return (double)((items + sms - 1) / sms) * c->n_sft * 1.44e-6;
+        return (double)items * c->n_sft / sms * 1.44e-6;
     };
     const double rate = L == 1 ? 2.7e11 : c->n_fdot <= 2 ? 4.6e11 : 5.6e11;
     const double t_other = (double)c->n_sky * c->n_fdot * c->n_f * c->n_sft / rate;
@@ -546,13 +547,17 @@ void choose_tc(fstat_ctx* c, int P, int L, bool found, Plan& pl) {
     const std::vector<TcSky> sky = tc_sky(c);
     for (int rt = kTcRows; rt >= 32 && t_tc(rt) <= 0.92 * t_other; rt /= 2) {
         double spread = tc_spread_bins(c, sky, rps, rt, nullptr);
+        bool nat = true;
         c->perm_on_device = 0;
-        std::vector<int> order = tc_neighbour_order(sky, (double)rt / rps);
-        const double q = tc_spread_bins(c, sky, rps, rt, &order);
-        const bool nat = spread <= q;
-        if (!nat) {
-            spread = q;
-            c->tc_order = std::move(order);
+        for (const double length : {1.0, 0.7, 1.4}) {   // one outlying tile decides: other strips may do without it
+            std::vector<int> order = tc_neighbour_order(sky, (double)rt / rps, length);
+            const double q = tc_spread_bins(c, sky, rps, rt, &order);
+            if (q < spread) {
+                spread = q;
+                nat = false;
+                c->tc_order = std::move(order);
+            }
+            if (spread <= kTcMaxSpread) break;
         }
         if (spread > kTcMaxSpread) continue;
         pl.tc = true;
@@ -1595,7 +1600,8 @@ int ensure_tables(fstat_ctx* c, cudaStream_t s) {
         xoff = (xoff + 4 + 3) & ~3;
         const int n_blk = (n_pos + 8 + 3) / 4;
         if ((rc = grow(c, &c->d_tcs, c->cap_tcs,
-                       (size_t)std::min(c->plan.tc_tiles * c->plan.tc_colb, current_sm_count()) * 2 * kTcRows * kTcCols)) !=
+                       (size_t)tc_blocks(c->plan.tc_tiles, c->plan.tc_colb, c->n_sft, current_sm_count()) * kTcSlots * kTcRows *
+                           kTcCols)) !=
             FSTAT_OK)
             return rc;
         if (c->gt_dirty || c->gt_nblk != n_blk || c->gt_xoff != xoff) {
@@ -1808,7 +1814,7 @@ int fstat_compute(fstat_ctx* c, void* cuda_stream) {
     cudaError_t e = launch_dir(c, dirichlet_params(c), c->plan.grid, s);
     if (e != cudaSuccess) return fail(c, FSTAT_ECUDA, "Dirichlet launch: %s", cudaGetErrorString(e));
     CUDA_TRY(c, cudaEventRecord(c->ev_c[slot], s));
-    c->launches += 2;   // timing + Dirichlet
+    c->launches += 1 + (c->plan.tc ? tc_launches(tc_params(c)) : 1);   // timing + Dirichlet
     if ((rc = enqueue_topk(c, s)) != FSTAT_OK) return rc;
     CUDA_TRY(c, cudaEventRecord(c->ev_d[slot], s));
     c->n_timed++;
@@ -2331,7 +2337,7 @@ int enqueue_batch(fstat_ctx* c, const std::vector<int>& order, const std::vector
         if (e != cudaSuccess) return fail(c, FSTAT_ECUDA, "batch Dirichlet launch: %s", cudaGetErrorString(e));
         stamp_kernel<<<1, 1, 0, s>>>(c->d_done + k);
         CUDA_TRY(c, cudaGetLastError());
-        c->launches += 2;
+        c->launches += 1 + tc_launches(tc_params(w));
     }
     for (size_t g = 1; g < groups.size(); ++g) CUDA_TRY(c, cudaStreamWaitEvent(s, c->side_events[g], 0));
     for (fstat_ctx* w : c->wus) {

@@ -17,7 +17,8 @@
 // A0 = A0h + A0l, products hh + hl + lh (2^-22 relative, the FP32 rounding
 // level); A1, A2 carry the drift (at most 1e-2 of the sum) and take one FP16
 // term each.  Measured against FP64 on random bins: rms error 7.9e-7 of the
-// rms bin at the largest Doppler drift, against 1.8e-6 for the sinc polynomial.
+// rms bin at the largest Doppler drift, against 1.8e-6 for the sinc polynomial;
+// 2F of whole searches 0.7e-6 against 1.7 to 1.9e-6.
 //
 // X as a matrix of shifted rows (B[c][k] = X[c + k]) is stored once per SFT in
 // 128-byte core matrices G[m] = { row i < 4: Re X[4m+i .. 4m+i+7], row 4 + i:
@@ -25,8 +26,8 @@
 // product is G[n + 2k], so overlapping descriptors (strides 128 and 256 bytes)
 // read the whole operand from 32 bytes a position and no row is ever copied.
 //
-// A block (one per SM, persistent over tiles of 128 rows x 64 columns) is a
-// pipeline of warps joined by mbarriers, over the SFTs:
+// A block (one per SM, persistent over its run of tiles of 128 rows x 64 columns
+// and SFTs, see block_first) is a pipeline of warps joined by mbarriers, over the SFTs:
 //   row constants (2 warps, two rows a lane, up to 8 SFTs ahead): khat and phase
 //     bases, kappa, the rows whose windows jump (below);
 //   copies (1 warp, 3 SFTs ahead): the window of core matrices that covers all
@@ -36,17 +37,18 @@
 //   products (1 warp): 5 tcgen05.mma per 16 positions into one of two
 //     accumulators in tensor memory;
 //   sums (8 warps: thread = row x 32 columns): window sums from tensor memory,
-//     twiddle, Fa and Fb in registers over all SFTs, then 2F.
+//     twiddle, Fa and Fb in registers, added up in tensor memory every 64 SFTs,
+//     then 2F.
 // A row whose window start jumps inside its 64 columns (khat crosses an
 // integer: about 64 eps of the (row, SFT)) has the two taps by which the windows
 // differ added by the copying warp into a per-block scratch of Fa, Fb.
 //
 // Bound: instruction issue (56 % active, 6750 warp instructions an SFT of 8192
 // pairs: 40 % sums, 40 % weights) with the latency of the stages; tensor pipe
-// 21 %, FMA pipes 43 %.  4000 sky x 1800 f x 10 spindowns x 2400 SFTs:
-// 198 ms (8.7e11 pairs/s) against 293 ms for the sinc ring; 2048 sky x 900 f x 1
-// x 1600: 4.6 against 6.9 ms; the 1/8-bin patch 2048 sky x 256 f: 2.3 against
-// 3.1 ms.  What it took, on 4000 sky x 640 f x 600 SFTs (ring 26 ms): one thread
+// 21 %, FMA pipes 43 %.  Against the sinc ring: 4000 sky x 1800 f x 10 spindowns x
+// 2400 SFTs 203 ms (8.5e11 pairs/s) against 293; 250 x 1733 x 7 x 2302, FP16 bins,
+// 217 Hz 9.1 against 15.7 ms; 2048 x 900 x 1 x 1600 4.1 against 6.9; the 1/8-bin
+// patch 2048 x 256 2.1 against 3.1.  What it took, on 4000 sky x 640 f x 600 SFTs (ring 26 ms): one thread
 // issuing copies and products beside its weights 55 ms; a warp of its own for
 // them, operands in uniform registers 22; code that fits the instruction caches
 // (rolled loops, short waits) and 8 weight warps 18.6; three operand buffers
@@ -71,6 +73,10 @@ constexpr uint32_t kAGroup = kRows * 32;                       // one weight arr
 constexpr uint32_t kABytes = 36 * kAGroup;                     // weight buffers: three of 3 groups x 4 arrays, or two of 4
 constexpr uint32_t kBlk = 256;                                 // core matrices of one 4-position block: high, low part
 constexpr uint32_t kXStage = kTcBlkMax * kBlk, kYStage = (kTcBlkMax - 1) * kBlk;
+// Fa, Fb go from registers into sums in tensor memory every kFlush SFTs: their
+// rounding grows with the root of a register sum's length (2F error against FP64:
+// 1.1e-6 without, 0.65e-6 with, 1600 to 2400 SFTs; no change in time).
+constexpr int kFlush = 64;
 constexpr int kStages = 4, kAhead = 3, kRing = 8;              // SFT stages, SFTs copied ahead, row-constant slots
 constexpr uint32_t kOffX = kABytes;
 constexpr uint32_t kOffY = kOffX + kStages * kXStage;
@@ -144,6 +150,14 @@ __device__ __forceinline__ void tmem_ld16(uint32_t addr, float (&v)[16]) {
           "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
         : "r"(addr));
 }
+__device__ __forceinline__ void tmem_st16(uint32_t addr, const float (&v)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15};" ::"f"(v[0]),
+        "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]), "f"(v[10]),
+        "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15]), "r"(addr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // the loaded registers pass through the wait, so nothing uses them before it
 __device__ __forceinline__ void tmem_wait16(float (&v)[16]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
@@ -284,6 +298,69 @@ __device__ __forceinline__ void put_weights(unsigned char* A, uint32_t arr, int 
 
 __device__ __forceinline__ void prefetch_l1(const void* q) { asm volatile("prefetch.global.L1 [%0];" ::"l"(q)); }
 
+// The steps (tile x column block, SFT), SFTs fastest, are dealt to the blocks in
+// equal runs, so that the last wave of tiles is no emptier than the others (2048 x
+// 900 x 1600, 240 tiles on 152 SMs: 5.2 -> 4.6 ms with the search's other kernels).  A
+// run starts and ends inside a tile: its first and last segment may hold part of
+// the SFTs.  They leave their sums in the scratch, in slot 0 (first segment) and
+// slots 1, 2 in turn (the others), for finish_kernel.
+constexpr int kScr = kRows * kCols, kSlots = kTcSlots;
+__device__ __forceinline__ long long block_first(const TcParams& p, unsigned b, unsigned blocks) {
+    return (long long)p.n_tiles * p.n_colb * p.n_sft * b / blocks;
+}
+// This block's first step, computed where it is used: the sum warps have no
+// register to keep it in.
+__device__ __forceinline__ long long run_first(const TcParams& p) {
+    unsigned b = blockIdx.x;
+    asm volatile("" : "+r"(b));
+    return block_first(p, b, gridDim.x);
+}
+__device__ __forceinline__ int seg_slot(int seg) { return seg == 0 ? 0 : 2 - (seg & 1); }
+
+// Where the 2F of a tile's row go: out[j], j < n_live (0: row of padding).
+struct RowOut {
+    float* out;
+    float4 cm;
+    int u, n_live;
+};
+__device__ __forceinline__ RowOut row_out(const TcParams& p, int item, int row) {
+    const int gr = (item % p.n_tiles) * p.rt + row;
+    const bool live = row < p.rt && gr < p.n_sky * p.rps;
+    const int place = (live ? gr : 0) / p.rps, rr = (live ? gr : 0) - place * p.rps;
+    const int d = rr / p.n_sub, sky = p.perm ? p.perm[place] : place;
+    return RowOut{p.twoF + ((size_t)sky * p.n_fdot + d) * p.n_f, p.comb[sky], rr - d * p.n_sub, live ? p.n_f : 0};
+}
+__device__ __forceinline__ float two_f(float4 cm, float4 F) {
+    const float f = cm.x * fmaf(F.x, F.x, F.y * F.y) + cm.y * fmaf(F.z, F.z, F.w * F.w) + cm.z * fmaf(F.x, F.z, F.y * F.w);
+    return fmaxf(f, 0.0f);
+}
+
+// 2F of the tiles whose SFTs were shared by several blocks: block x takes the
+// tile that block x of the sums (of `blocks`) began and did not end, adds the
+// parts in SFT order, y taking a share of the rows.
+__global__ void __launch_bounds__(256) finish_kernel(const TcParams p, int blocks) {
+    const int b = blockIdx.x;
+    const long long t0 = block_first(p, b, blocks), t1 = block_first(p, b + 1, blocks);
+    if (t1 <= t0) return;
+    const int item = (int)((t1 - 1) / p.n_sft);
+    const long long first = (long long)item * p.n_sft, end = first + p.n_sft;
+    if (first < t0 || end <= t1) return;   // begun by another block, or whole
+    const int slot = seg_slot(item - (int)(t0 / p.n_sft));
+    const int c0 = (item / p.n_tiles) * kCols;
+    const int col = threadIdx.x & (kCols - 1);
+    for (int row = blockIdx.y * 4 + (threadIdx.x >> 6); row < kRows; row += gridDim.y * 4) {
+        const RowOut o = row_out(p, item, row);
+        const int j = p.n_sub * (c0 + col) + o.u;
+        if (j >= o.n_live) continue;
+        float4 F = __ldcg(p.scratch + ((size_t)b * kSlots + slot) * kScr + row * kCols + col);
+        for (int q = b + 1; q < blocks && block_first(p, q, blocks) < end; ++q) {
+            const float4 x = __ldcg(p.scratch + (size_t)q * kSlots * kScr + row * kCols + col);
+            F = make_float4(F.x + x.x, F.y + x.y, F.z + x.z, F.w + x.w);
+        }
+        o.out[j] = two_f(o.cm, F);
+    }
+}
+
 __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -299,12 +376,16 @@ __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParam
     auto t_full = [&](int i) { return bar(29 + (i & 1)); };        // [2] tile's window jumps all in place
     auto x_free = [&](unsigned n) { return bar(31 + (n & 3)); };   // [4] SFT's bins read by the products and the window jumps
     const uint32_t fin = bar(35);                                  // last products done
-    uint32_t* ctrl = reinterpret_cast<uint32_t*>(smem + kOffCtrl); // [0] tensor-memory address
+    uint32_t* ctrl = reinterpret_cast<uint32_t*>(smem + kOffCtrl); // [0] tensor-memory address, [1] steps
     if (warp == 16) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(sb + kOffCtrl) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(sb + kOffCtrl) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    const long long t0 = block_first(p, blockIdx.x, gridDim.x);
+    const unsigned n_steps = (unsigned)(block_first(p, blockIdx.x + 1, gridDim.x) - t0);
+    const int item0 = (int)(t0 / p.n_sft), sft0 = (int)(t0 - (long long)item0 * p.n_sft);   // the run's first step
     if (tid == 0) {
+        ctrl[1] = n_steps;
         for (int i = 0; i < 4; ++i) {
             mbar_init(x_full(i), 1);
             mbar_init(x_free(i), 2);
@@ -323,16 +404,15 @@ __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParam
         mbar_init(fin, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // the block's scratch of window-jump corrections, one per tile parity
-    constexpr int kScr = kRows * kCols;
-    float4* scratch = p.scratch + (size_t)blockIdx.x * 2 * kScr;
-    for (int i = tid; i < 2 * kScr; i += kThreads) __stcg(scratch + i, make_float4(0.f, 0.f, 0.f, 0.f));
+    // the block's scratch of window-jump corrections (slot of a segment: seg_slot)
+    float4* scratch = p.scratch + (size_t)blockIdx.x * kSlots * kScr;
+    const int n_segs = (int)((sft0 + (long long)n_steps - 1) / p.n_sft) + 1;
+    for (int i = tid; i < min(n_segs, kSlots) * kScr; i += kThreads) __stcg(scratch + i, make_float4(0.f, 0.f, 0.f, 0.f));
     __threadfence();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = ctrl[0];
-    const int n_items = p.n_tiles * p.n_colb;
     const int row = tid & 127;
     int2* win = reinterpret_cast<int2*>(smem + kOffWin);   // [8] first block, position groups of an SFT
     int2* mm = reinterpret_cast<int2*>(smem + kOffMM);     // [8][2 warps] lowest and highest first position of the rows
@@ -344,92 +424,93 @@ __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParam
     // a give-up is uniform over the warp, whose later steps are warp-wide
     auto wait = [&](uint32_t at, unsigned phase) { return __all_sync(0xffffffffu, wait_bar(at, phase & 1u)) != 0; };
     bool ok = true;
-    unsigned n = 0;   // SFTs so far over all tiles of the block
+    unsigned n = 0;   // steps so far
 
     if (warp < 8) {
         // ---- weights: thread = row, warpgroup = half of the taps ----------------------
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kGenRegs));
         int buf = 0;              // weight buffer of SFT n
         unsigned turn = 0;        // its uses so far
-        for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-            for (int s = 0; s < p.n_sft; ++s, ++n) {
-                ok = wait(r_full(n), n >> 3) && wait(x_full(n), n >> 2) &&      // window known
-                     (turn == 0 || wait(a_free(buf), turn - 1));
-                if (!ok) break;
-                const float4 w = W4[(n & 7) * kRows + row];
-                const int2 wn = win[n & 7];
-                int sh = __float_as_int(w.z) - 4 * wn.x;
-                if (sh < 0 || sh > 16 * wn.y - 16) {   // cannot happen with the planner's bounds
-                    atomicOr(p.err, 1);
-                    sh = max(0, min(sh, 16 * wn.y - 16));
-                }
-                put_weights(smem + buf * 4 * a_arr + (warp >> 2) * (kAGroup / 2) + (row >> 3) * 128 + (row & 7) * 16, a_arr,
-                            warp >> 2, sh, wn.y, w.x, w.y);
-                if (++buf == n_buf) {
-                    buf = 0;
-                    ++turn;
-                }
-                ok = n < 2 || wait(d_full(n), (n - 2) >> 1);   // the q X buffer is read
-                if (!ok) break;
-                // q X and q^2 X (first FP16 part only), 16 bytes a thread
-                if (tid < (14 + 4 * wn.y) * 8) {
-                    const uint32_t o = (uint32_t)(tid >> 3) * kBlk + (uint32_t)(tid & 7) * 16;
-                    const uint4 v = *reinterpret_cast<const uint4*>(smem + kOffX + (n & 3) * kXStage + o);
-                    const float q0 = (float)(4 * (tid >> 3) + (tid & 3) - 48) * 0.015625f;
-                    const __half2 q = __floats2half2_rn(q0, q0 + 0.015625f);
-                    const uint32_t in[4] = {v.x, v.y, v.z, v.w};
-                    uint32_t y[4], z[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const __half2 qe = __hadd2(q, __floats2half2_rn(0.03125f * e, 0.03125f * e));   // exact
-                        const __half2 yy = __hmul2(*reinterpret_cast<const __half2*>(&in[e]), qe);
-                        const __half2 zz = __hmul2(yy, qe);
-                        y[e] = *reinterpret_cast<const uint32_t*>(&yy);
-                        z[e] = *reinterpret_cast<const uint32_t*>(&zz);
-                    }
-                    unsigned char* Y = smem + kOffY + (n & 1) * kYStage + o;
-                    *reinterpret_cast<uint4*>(Y) = make_uint4(y[0], y[1], y[2], y[3]);
-                    *reinterpret_cast<uint4*>(Y + 128) = make_uint4(z[0], z[1], z[2], z[3]);
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) mbar_arrive(a_full(n));
+        for (; n < ctrl[1]; ++n) {
+            ok = wait(r_full(n), n >> 3) && wait(x_full(n), n >> 2) &&      // window known
+                 (turn == 0 || wait(a_free(buf), turn - 1));
+            if (!ok) break;
+            const float4 w = W4[(n & 7) * kRows + row];
+            const int2 wn = win[n & 7];
+            int sh = __float_as_int(w.z) - 4 * wn.x;
+            if (sh < 0 || sh > 16 * wn.y - 16) {   // cannot happen with the planner's bounds
+                atomicOr(p.err, 1);
+                sh = max(0, min(sh, 16 * wn.y - 16));
             }
+            put_weights(smem + buf * 4 * a_arr + (warp >> 2) * (kAGroup / 2) + (row >> 3) * 128 + (row & 7) * 16, a_arr,
+                        warp >> 2, sh, wn.y, w.x, w.y);
+            if (++buf == n_buf) {
+                buf = 0;
+                ++turn;
+            }
+            ok = n < 2 || wait(d_full(n), (n - 2) >> 1);   // the q X buffer is read
+            if (!ok) break;
+            // q X and q^2 X (first FP16 part only), 16 bytes a thread
+            if (tid < (14 + 4 * wn.y) * 8) {
+                const uint32_t o = (uint32_t)(tid >> 3) * kBlk + (uint32_t)(tid & 7) * 16;
+                const uint4 v = *reinterpret_cast<const uint4*>(smem + kOffX + (n & 3) * kXStage + o);
+                const float q0 = (float)(4 * (tid >> 3) + (tid & 3) - 48) * 0.015625f;
+                const __half2 q = __floats2half2_rn(q0, q0 + 0.015625f);
+                const uint32_t in[4] = {v.x, v.y, v.z, v.w};
+                uint32_t y[4], z[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const __half2 qe = __hadd2(q, __floats2half2_rn(0.03125f * e, 0.03125f * e));   // exact
+                    const __half2 yy = __hmul2(*reinterpret_cast<const __half2*>(&in[e]), qe);
+                    const __half2 zz = __hmul2(yy, qe);
+                    y[e] = *reinterpret_cast<const uint32_t*>(&yy);
+                    z[e] = *reinterpret_cast<const uint32_t*>(&zz);
+                }
+                unsigned char* Y = smem + kOffY + (n & 1) * kYStage + o;
+                *reinterpret_cast<uint4*>(Y) = make_uint4(y[0], y[1], y[2], y[3]);
+                *reinterpret_cast<uint4*>(Y + 128) = make_uint4(z[0], z[1], z[2], z[3]);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(a_full(n));
         }
     } else if (warp >= 16) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kAuxRegs));
         if (warp == 16) {
             // ---- products ------------------------------------------------------------------------
             int buf = 0;
-            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-                for (int s = 0; s < p.n_sft; ++s, ++n) {
-                    ok = wait(a_full(n), n >> 1) && (n < 2 || wait(d_free(n), (n - 2) >> 1));
-                    if (!ok) break;
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const int gk = win[n & 7].y;
-                    const uint32_t dst = tmem + (n & 1) * (2 * kCols);
-                    const uint32_t a = desc_lo(sb + buf * 4 * a_arr, kAGroup / 2), arr = a_arr / 16;
-                    const uint32_t x = desc_lo(sb + kOffX + (n & 3) * kXStage, 2 * kBlk);
-                    const uint32_t y = desc_lo(sb + kOffY + (n & 1) * kYStage, 2 * kBlk);
+            for (; n < ctrl[1]; ++n) {
+                ok = wait(a_full(n), n >> 1) && (n < 2 || wait(d_free(n), (n - 2) >> 1));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const int gk = win[n & 7].y;
+                const uint32_t dst = tmem + (n & 1) * (2 * kCols);
+                const uint32_t a = desc_lo(sb + buf * 4 * a_arr, kAGroup / 2), arr = a_arr / 16;
+                const uint32_t x = desc_lo(sb + kOffX + (n & 3) * kXStage, 2 * kBlk);
+                const uint32_t y = desc_lo(sb + kOffY + (n & 1) * kYStage, 2 * kBlk);
+// the accumulator is cut off, not rounded, at each product: the small
+                // terms go first, so that few products see its full size (hh first: 2F
+                // 5e-7 too small on average).  Offsets in 16-byte units of the start address.
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {   // offsets in 16-byte units of the start address
-                        if (q < gk) {
-                            const uint32_t aq = a + q * (kAGroup / 16), xq = x + q * (4 * kBlk / 16), yq = y + q * (4 * kBlk / 16);
-                            mma_issue(dst, aq, xq, q);
-                            mma_issue(dst, aq, xq + 128 / 16, 1u);
-                            mma_issue(dst, aq + arr, xq, 1u);
-                            mma_issue(dst, aq + 2 * arr, yq, 1u);
-                            mma_issue(dst, aq + 3 * arr, yq + 128 / 16, 1u);
-                        }
+                for (int q = 0; q < 4; ++q) {
+                    if (q < gk) {
+                        const uint32_t aq = a + q * (kAGroup / 16), xq = x + q * (4 * kBlk / 16), yq = y + q * (4 * kBlk / 16);
+                        mma_issue(dst, aq + 3 * arr, yq + 128 / 16, q);
+                        mma_issue(dst, aq + 2 * arr, yq, 1u);
+                        mma_issue(dst, aq, xq + 128 / 16, 1u);
+                        mma_issue(dst, aq + arr, xq, 1u);
                     }
-                    if (lane == 0) {
-                        mma_commit(d_full(n));
-                        mma_commit(a_free(buf));
-                        mma_commit(x_free(n));
-                    }
-                    __syncwarp();
-                    buf = buf + 1 == n_buf ? 0 : buf + 1;
                 }
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (q < gk) mma_issue(dst, a + q * (kAGroup / 16), x + q * (4 * kBlk / 16), 1u);
+                if (lane == 0) {
+                    mma_commit(d_full(n));
+                    mma_commit(a_free(buf));
+                    mma_commit(x_free(n));
+                }
+                __syncwarp();
+                buf = buf + 1 == n_buf ? 0 : buf + 1;
             }
             if (lane == 0) mma_commit(fin);
             __syncwarp();
@@ -463,42 +544,44 @@ __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParam
                 if (p.stop < 0 || s < p.stop) issued = q + 1;
                 return true;
             };
-            int item_no = 0;
-            for (int s = 0; s < kAhead && ok; ++s) ok = copy_sft(s, (unsigned)s);
-            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++item_no) {
-                float4* scr = scratch + (item_no & 1) * kScr;
-                for (int s = 0; s < p.n_sft; ++s, ++n) {
-                    const int nxt = s + kAhead;
-                    if (nxt < p.n_sft) ok = copy_sft(nxt, n + kAhead);
-                    else if (item + (int)gridDim.x < n_items) ok = copy_sft(nxt - p.n_sft, n + kAhead);
-                    ok = ok && wait(x_full(n), n >> 2);
-                    if (!ok) break;
-                    const int2 wn = win[n & 7];
-                    const unsigned char* X = smem + kOffX + (n & 3) * kXStage;
+            int seg = 0, s = sft0, nxt = s;   // SFT of this step, of the next copy
+            for (unsigned q = 0; q < kAhead && q < n_steps && ok; ++q) {
+                ok = copy_sft(nxt, q);
+                nxt = nxt + 1 == p.n_sft ? 0 : nxt + 1;
+            }
+            for (; n < n_steps && ok; ++n) {
+                float4* scr = scratch + seg_slot(seg) * kScr;
+                if (n + kAhead < n_steps) ok = copy_sft(nxt, n + kAhead);
+                nxt = nxt + 1 == p.n_sft ? 0 : nxt + 1;
+                ok = ok && wait(x_full(n), n >> 2);
+                if (!ok) break;
+                const int2 wn = win[n & 7];
+                const unsigned char* X = smem + kOffX + (n & 3) * kXStage;
 #pragma unroll 1
-                    for (int r = 0; r < 4; ++r) {
-                        uint32_t ev = *reinterpret_cast<const uint32_t*>(smem + kOffEv + (n & 7) * 16 + 4 * r);
-                        while (ev) {   // the lanes take the columns
-                            const int src = 32 * r + __ffs(ev) - 1;
-                            ev &= ev - 1;
-                            const float4 u = W4[(n & 7) * kRows + src], e4 = P4[(n & 7) * kRows + src];
-                            const float b = B1[(n & 7) * kRows + src];
-                            const int sh = max(0, min(__float_as_int(u.z) - 4 * wn.x, 16 * wn.y - 16));
+                for (int r = 0; r < 4; ++r) {
+                    uint32_t ev = *reinterpret_cast<const uint32_t*>(smem + kOffEv + (n & 7) * 16 + 4 * r);
+                    while (ev) {   // the lanes take the columns
+                        const int src = 32 * r + __ffs(ev) - 1;
+                        ev &= ev - 1;
+                        const float4 u = W4[(n & 7) * kRows + src], e4 = P4[(n & 7) * kRows + src];
+                        const float b = B1[(n & 7) * kRows + src];
+                        const int sh = max(0, min(__float_as_int(u.z) - 4 * wn.x, 16 * wn.y - 16));
 #pragma unroll 2
-                            for (int c = lane; c < kCols; c += 32)
-                                window_jump(X, 14 + 4 * wn.y, sh, u.x, u.y, __float_as_uint(e4.x), __float_as_uint(e4.y), u.w,
-                                            b, c, scr + src * kCols);
-                        }
-                    }
-                    const bool last = s + 1 == p.n_sft;
-                    if (last) __threadfence();
-                    __syncwarp();
-                    if (lane == 0) {
-                        mbar_arrive(r_free(n));
-                        mbar_arrive(x_free(n));
-                        if (last) mbar_arrive(t_full(item_no));
+                        for (int c = lane; c < kCols; c += 32)
+                            window_jump(X, 14 + 4 * wn.y, sh, u.x, u.y, __float_as_uint(e4.x), __float_as_uint(e4.y), u.w,
+                                        b, c, scr + src * kCols);
                     }
                 }
+                const bool last = s + 1 == p.n_sft || n + 1 == n_steps;
+                if (last) __threadfence();
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(r_free(n));
+                    mbar_arrive(x_free(n));
+                    if (last) mbar_arrive(t_full(seg));
+                }
+                seg += last;
+                s = s + 1 == p.n_sft ? 0 : s + 1;
             }
             if (!ok) {
                 // copies still in flight land before the block retires
@@ -507,7 +590,9 @@ __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParam
         } else {
             // ---- row constants: two rows a thread, up to kRing SFTs ahead --------------------
             const int rw0 = (warp - 18) * 64 + lane;   // the thread's rows rw0 and rw0 + 32
-            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+            int s0 = sft0;
+            for (int item = item0; n < n_steps && ok; ++item, s0 = 0) {
+                const int s1 = (int)min((unsigned)p.n_sft, s0 + (n_steps - n));
                 const int tile = item % p.n_tiles, c0 = (item / p.n_tiles) * kCols;
                 auto row_of = [&](int rw, int& place, int& d, int& j0) {
                     const int g = min(tile * p.rt + min(rw, p.rt - 1), p.n_sky * p.rps - 1);
@@ -519,7 +604,7 @@ __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParam
                 int place0, d0, j00, place1, d1, j01;
                 row_of(rw0, place0, d0, j00);
                 row_of(rw0 + 32, place1, d1, j01);
-                for (int s = 0; s < p.n_sft; ++s, ++n) {
+                for (int s = s0; s < s1; ++s, ++n) {
                     if (n >= kRing) ok = wait(r_free(n), (n - kRing) >> 3);
                     if (!ok) break;
                     const float isc = __ldg(p.inv_scale + s);
@@ -572,12 +657,32 @@ __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParam
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSumRegs));
         const int h = (warp - 8) >> 2;
         const uint32_t tbase = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 64u * h;
-        int item_no = 0;
-        for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++item_no) {
+        const uint32_t sums = tbase + 4 * kCols + 64u * h;   // columns 256 + 128 h: the thread's 32 columns of Fa, Fb
+        int seg = 0;
+        for (; n < ctrl[1] && ok; ++seg) {
+            const unsigned end = min(ctrl[1], n + p.n_sft - (unsigned)((run_first(p) + n) % p.n_sft));
             float2 far[16], fai[16], fbr[16], fbi[16];   // column pairs
+            auto clear = [&](int i) { far[i] = fai[i] = fbr[i] = fbi[i] = make_float2(0.f, 0.f); };
+            // columns 4k .. 4k + 3 added to v
+            auto add4 = [&](int k, float (&v)[16]) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) far[i] = fai[i] = fbr[i] = fbi[i] = make_float2(0.f, 0.f);
-            for (int s = 0; s < p.n_sft; ++s, ++n) {
+                for (int e = 0; e < 2; ++e) {
+                    const int i = 2 * k + e;
+                    v[2 * e] += far[i].x, v[2 * e + 1] += far[i].y;
+                    v[4 + 2 * e] += fai[i].x, v[5 + 2 * e] += fai[i].y;
+                    v[8 + 2 * e] += fbr[i].x, v[9 + 2 * e] += fbr[i].y;
+                    v[12 + 2 * e] += fbi[i].x, v[13 + 2 * e] += fbi[i].y;
+                }
+            };
+            float zero[16] = {};
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                clear(2 * k);
+                clear(2 * k + 1);
+                tmem_st16(sums + 16 * k, zero);
+            }
+            tmem_wait_st();
+            for (; n < end; ++n) {
                 ok = wait(r_full(n), n >> 3);
                 if (!ok) break;
                 const float4 p4 = P4[(n & 7) * kRows + row];
@@ -634,35 +739,49 @@ __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParam
                     mbar_arrive(d_free(n));
                     mbar_arrive(r_free(n));
                 }
+                if ((n & (kFlush - 1)) == kFlush - 1) {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        float u[16];
+                        tmem_ld16(sums + 16 * k, u);
+                        tmem_wait16(u);
+                        add4(k, u);
+                        clear(2 * k);
+                        clear(2 * k + 1);
+                        tmem_st16(sums + 16 * k, u);
+                    }
+                    tmem_wait_st();
+                }
             }
-            if (ok) ok = wait(t_full(item_no), (unsigned)item_no >> 1);
+            if (ok) ok = wait(t_full(seg), (unsigned)seg >> 1);
             if (!ok) break;
-            // 2F of the row's columns, window-jump corrections added; the scratch is left at zero
-            const int tile = item % p.n_tiles, c0 = (item / p.n_tiles) * kCols + 32 * h;
-            const int gr = tile * p.rt + row;
-            const bool live = row < p.rt && gr < p.n_sky * p.rps;
-            const int place = (live ? gr : 0) / p.rps, rr = (live ? gr : 0) - place * p.rps;
-            const int d = rr / p.n_sub, u = rr - d * p.n_sub;
-            const int sky = p.perm ? p.perm[place] : place;
-            const float4 cm = p.comb[sky];
-            float* out = p.twoF + ((size_t)sky * p.n_fdot + d) * p.n_f;
-            float4* rs = scratch + (item_no & 1) * kScr + row * kCols + 32 * h;
+            // 2F of the row's columns, window-jump corrections added, and the scratch left
+            // at zero; of a part of the SFTs, the sums instead of it
+            const long long first = run_first(p), t = first + n;
+            const int item = (int)((t - 1) / p.n_sft);
+            const long long begin = (long long)item * p.n_sft;
+            const bool whole = begin >= first && t == begin + p.n_sft;
+            const RowOut o = row_out(p, item, row);
+            const int j0 = p.n_sub * ((item / p.n_tiles) * kCols + 32 * h) + o.u;
+            float4* rs = scratch + seg_slot(seg) * kScr + row * kCols + 32 * h;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {   // eight columns at a time: their loads fly together
-                float4 x[8];
+            for (int q = 0; q < 8; ++q) {   // four columns at a time: their loads fly together
+                float4 x[4];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) x[e] = __ldcg(rs + 8 * q + e);
+                for (int e = 0; e < 4; ++e) x[e] = __ldcg(rs + 4 * q + e);
+                float u[16];
+                tmem_ld16(sums + 16 * q, u);
+                tmem_wait16(u);
+                add4(q, u);
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const int i = 4 * q + (e >> 1);
-                    const float ar = (e & 1 ? far[i].y : far[i].x) + x[e].x, ai = (e & 1 ? fai[i].y : fai[i].x) + x[e].y;
-                    const float br = (e & 1 ? fbr[i].y : fbr[i].x) + x[e].z, bi = (e & 1 ? fbi[i].y : fbi[i].x) + x[e].w;
-                    const int j = p.n_sub * (c0 + 8 * q + e) + u;
-                    const float f = cm.x * fmaf(ar, ar, ai * ai) + cm.y * fmaf(br, br, bi * bi) +
-                                    cm.z * fmaf(ar, br, ai * bi);
-                    if (live && j < p.n_f) out[j] = fmaxf(f, 0.0f);
-                    if (x[e].x != 0.f || x[e].y != 0.f || x[e].z != 0.f || x[e].w != 0.f)
-                        __stcg(rs + 8 * q + e, make_float4(0.f, 0.f, 0.f, 0.f));
+                for (int e = 0; e < 4; ++e) {
+                    const int c = 4 * q + e;
+                    const bool hot = x[e].x != 0.f || x[e].y != 0.f || x[e].z != 0.f || x[e].w != 0.f;
+                    x[e] = make_float4(x[e].x + u[e], x[e].y + u[4 + e], x[e].z + u[8 + e], x[e].w + u[12 + e]);
+                    const int j = j0 + p.n_sub * c;
+                    if (whole && j < o.n_live) o.out[j] = two_f(o.cm, x[e]);
+                    if (whole) x[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (hot || !whole) __stcg(rs + c, x[e]);
                 }
             }
             __threadfence();   // the zeros are in place before the scratch's next tile
@@ -673,7 +792,7 @@ __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParam
     __syncthreads();
     if (warp == 16) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
     }
 }
 
@@ -742,11 +861,24 @@ cudaError_t launch_tc_tables(const void* bins, int form, long long row, int n_sf
     return cudaGetLastError();
 }
 
+// One block an SM, but at least 32 steps a block where there are fewer tiles.
+int tc_blocks(int n_tiles, int n_colb, int n_sft, int sms) {
+    const long long items = (long long)n_tiles * n_colb;
+    return (int)std::min<long long>(sms, std::max(std::min<long long>(items, sms), items * n_sft / 32));
+}
+
+int tc_launches(const TcParams& p) {
+    const int grid = tc_blocks(p.n_tiles, p.n_colb, p.n_sft, current_sm_count());
+    return (long long)p.n_tiles * p.n_colb % grid == 0 ? 1 : 2;   // whole tiles only, or finish_kernel too
+}
+
 cudaError_t launch_dirichlet_tc(const TcParams& p, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(dirichlet_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
     if (e != cudaSuccess) return e;
-    const int grid = std::min(p.n_tiles * p.n_colb, current_sm_count());
+    const int grid = tc_blocks(p.n_tiles, p.n_colb, p.n_sft, current_sm_count());
     dirichlet_tc_kernel<<<grid, kThreads, kSmem, s>>>(p);
+    if ((e = cudaGetLastError()) != cudaSuccess || tc_launches(p) == 1) return e;
+    finish_kernel<<<dim3(grid, 8), 256, 0, s>>>(p, grid);
     return cudaGetLastError();
 }
 

@@ -199,6 +199,7 @@ __host__ __device__ inline RingSmem ring_smem(int stages, int w_tab, bool sinc =
 // kTcRows rows (sky point x spindown x sub-bin offset) x kTcCols columns (one
 // bin apart).
 constexpr int kTcRows = 128, kTcCols = 64;
+constexpr int kTcSlots = 3;        // scratch slots of a block (rows x columns of Fa, Fb)
 constexpr int kTcBlkMax = 31;      // 4-position blocks copied for the widest window
 constexpr int kTcMaxSpread = 45;   // bins between the lowest and highest window of a tile's rows
 struct TcParams {
@@ -211,7 +212,7 @@ struct TcParams {
     const float4* comb;            // [n_sky]
     const int* perm;               // sky point at each place of the grouping order, or null
     float* twoF;                   // [n_sky][n_fdot][n_f]
-    float4* scratch;               // [blocks][2][kTcRows][kTcCols]
+    float4* scratch;               // [blocks][kTcSlots][kTcRows][kTcCols]
     int* err;
     int n_sft, n_sky, n_fdot, n_f;
     int n_sub;                     // templates per bin: template j = n_sub * column + offset
@@ -302,6 +303,8 @@ cudaError_t launch_sinc_tables(const void* bins, int form, long long row, int n_
                                cudaStream_t s);
 cudaError_t launch_tc_tables(const void* bins, int form, long long row, int n_sft, int n_bins, int n_blk, int xoff,
                              unsigned char* gtab, float* inv_scale, cudaStream_t s);
+int tc_blocks(int n_tiles, int n_colb, int n_sft, int sms);   // blocks of the kernel
+int tc_launches(const TcParams& p);                            // kernels that launch_dirichlet_tc launches
 cudaError_t launch_dirichlet_tc(const TcParams& p, cudaStream_t s);
 cudaError_t launch_dirichlet_far(int v, const DirichletParams& p, int threads, size_t smem, long long grid,
                                  cudaStream_t s);

@@ -154,3 +154,39 @@ def test_batched_tensor_workunits_equal_single_launches(lib):
         assert np.all(done > 0) and np.all(done <= total * 1.001)
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("n_sky,sizes", [
+    (300, dict(n_sft=60, n_f=301, n_fdot=5, n_bins=340)),     # 60 tiles: two or three blocks a tile
+    (520, dict(n_sft=6, n_f=510, n_fdot=5, n_bins=550)),      # 168 tiles: most blocks start inside one
+    (1130, dict(n_sft=5, n_f=320, n_fdot=5, n_bins=360)),     # 225 tiles: runs of one and a half
+    (2400, dict(n_sft=4, n_f=320, n_fdot=5, n_bins=360)),     # 470 tiles: three or four segments, all scratch slots
+])
+def test_tiles_shared_by_blocks(lib, n_sky, sizes):
+    """Parts of a tile's SFTs on different blocks, against the direct form."""
+    w = _dense(n_sky, **sizes)
+    bins = O.inject(w.detectors, w.T, w.k_lo, w.injections, w.bank.t_ref)
+    got, _, flags, tiles = _run(lib, w, bins)
+    assert tiles["rows"] > 0 and flags == 0
+    again, _, _, _ = _run(lib, w, bins)
+    np.testing.assert_array_equal(got, again)     # the parts are added in one order
+    direct, _, _, none = _run(lib, w, bins, algo="direct")
+    assert none["rows"] == 0
+    assert np.all(np.abs(got.astype(np.float64) - direct) <= 2 * (REL * np.abs(direct) + ABS))
+
+
+@pytest.mark.parametrize("n_sky,f0", [(250, 217.0), (1500, 390.0)])
+def test_sparse_skies_at_high_frequency(lib, n_sky, f0):
+    """Tiles of far-apart sky points of both hemispheres over two months: the
+    planner's bound holds the windows (no range flag)."""
+    w = _dense(n_sky, n_sft=30, n_f=512, n_fdot=7, n_bins=760)
+    spread = [dataclasses.replace(d, t_start=w.bank.t_ref + (d.t_start - d.t_start[0]) * 5.2e6 / max(d.t_start[-1] - d.t_start[0], 1.0))
+            for d in w.detectors]
+    shift = int(round(f0 * w.T)) - int(round(w.bank.f0 * w.T))
+    bank = dataclasses.replace(w.bank, f0=w.bank.f0 + shift / w.T)
+    w = dataclasses.replace(w, detectors=spread, bank=bank, k_lo=w.k_lo + shift)
+    bins = [d.bins for d in w.detectors]
+    got, _, flags, tiles = _run(lib, w, bins)
+    direct, _, dflags, _ = _run(lib, w, bins, algo="direct")
+    assert tiles["rows"] > 0 and flags == dflags
+    assert np.all(np.abs(got.astype(np.float64) - direct) <= 2 * (REL * np.abs(direct) + ABS))

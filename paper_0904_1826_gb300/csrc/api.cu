@@ -538,7 +538,7 @@ void choose_tc(fstat_ctx* c, int P, int L, bool found, Plan& pl) {
     // where the steps are 1/8 bin (L = 1); smaller banks leave them slower.
     auto t_tc = [&](int rt) {
         const long long items = ((n_rows + rt - 1) / rt) * colb;
-        return (double)items * c->n_sft / sms * 1.44e-6;
+        return (double)items * c->n_sft / tc_blocks((int)((n_rows + rt - 1) / rt), (int)colb, c->n_sft, sms) * 1.44e-6;
     };
     const double rate = L == 1 ? 2.7e11 : c->n_fdot <= 2 ? 4.6e11 : 5.6e11;
     const double t_other = (double)c->n_sky * c->n_fdot * c->n_f * c->n_sft / rate;

@@ -878,7 +878,7 @@ cudaError_t launch_dirichlet_tc(const TcParams& p, cudaStream_t s) {
     const int grid = tc_blocks(p.n_tiles, p.n_colb, p.n_sft, current_sm_count());
     dirichlet_tc_kernel<<<grid, kThreads, kSmem, s>>>(p);
     if ((e = cudaGetLastError()) != cudaSuccess || tc_launches(p) == 1) return e;
-    finish_kernel<<<dim3(grid, 8), 256, 0, s>>>(p, grid);
+    finish_kernel<<<dim3(grid, 16), 256, 0, s>>>(p, grid);
     return cudaGetLastError();
 }
 

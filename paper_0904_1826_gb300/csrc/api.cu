@@ -125,6 +125,7 @@ struct fstat_ctx {
     // per-SFT frequency coverage (fstat_set_coverage)
     bool have_cov = false;
     int2* d_cov = nullptr;          // [n_sft] frequency-index range [x, y)
+    std::vector<int2> h_cov;        // the same, on the host
     float4* d_comb_j = nullptr;     // [n_sky][n_f] combine weights per frequency
     size_t cap_comb_j = 0;
     // stack-slide scratch (held by the first segment of a call)
@@ -519,12 +520,12 @@ std::vector<int> tc_neighbour_order(const std::vector<TcSky>& sky, double g, dou
 // Tensor-core form where it is the faster one.  It needs column steps of one
 // bin (n_sub = P / L templates a bin), a uniform spindown grid, at least 8 SFTs
 // (its blocks work up to 6 ahead) and windows of a tile's rows within
-// kTcMaxSpread bins; frequency coverage, Kahan sums, other D and explicit tile
-// or form requests keep the other forms.
+// kTcMaxSpread bins; Kahan sums, other D and explicit tile or form requests keep
+// the other forms.
 void choose_tc(fstat_ctx* c, int P, int L, bool found, Plan& pl) {
     pl.tc = false;
     const fstat_opts& o = c->opts0;
-    if (!found || P % L != 0 || !c->fdot_uniform || c->have_cov || c->n_sft < 8) return;
+    if (!found || P % L != 0 || !c->fdot_uniform || c->n_sft < 8) return;
     if (o.algo != FSTAT_ALGO_AUTO || o.tile_m > 0 || o.tile_warps > 0 || o.sft_chunk > 0) return;
     const int n_sub = P / L, rps = c->n_fdot * n_sub;
     const long long n_rows = (long long)c->n_sky * rps;
@@ -541,7 +542,13 @@ void choose_tc(fstat_ctx* c, int P, int L, bool found, Plan& pl) {
         return (double)items * c->n_sft / tc_blocks((int)((n_rows + rt - 1) / rt), (int)colb, c->n_sft, sms) * 1.44e-6;
     };
     const double rate = L == 1 ? 2.7e11 : c->n_fdot <= 2 ? 4.6e11 : 5.6e11;
-    const double t_other = (double)c->n_sky * c->n_fdot * c->n_f * c->n_sft / rate;
+    double pairs = (double)c->n_sky * c->n_fdot * c->n_f * c->n_sft;
+    if (c->have_cov) {   // the other forms skip an SFT that covers none of a thread's templates, this one masks it
+        double covered = 0.0;
+        for (const int2& v : c->h_cov) covered += std::max(0, std::min(v.y, c->n_f) - std::max(v.x, 0));
+        pairs *= covered / ((double)c->n_f * c->n_sft);
+    }
+    const double t_other = pairs / rate;
     if (n_rows > (1 << 28) || (n_rows / 32 + 1) * colb > (1 << 28) || t_other > 3000.0) return;   // 32-bit counters
     if (t_tc(kTcRows) > 0.92 * t_other) return;
     const std::vector<TcSky> sky = tc_sky(c);
@@ -1112,6 +1119,7 @@ int make_plan(fstat_ctx* c, Plan& out) {
     }
     if (!have) return fail(c, FSTAT_EINVAL, "no Dirichlet tile plan fits this template bank");
     out = best;
+    if (far_eligible(c) && c->have_cov) choose_tc(c, P, L, found, out);   // the rings take coverage at L = 2 only
     return FSTAT_OK;
 }
 
@@ -1318,6 +1326,7 @@ int fstat_set_coverage(fstat_ctx* c, const int32_t* j_lo, const int32_t* j_hi, i
     c->d_cov = nullptr;
     CUDA_TRY(c, cudaMalloc(&c->d_cov, (size_t)n_sft * sizeof(int2)));
     CUDA_TRY(c, cudaMemcpy(c->d_cov, h.data(), (size_t)n_sft * sizeof(int2), cudaMemcpyHostToDevice));
+    c->h_cov = std::move(h);
     c->have_cov = true;
     c->plan_valid = false;
     c->computed = false;
@@ -1735,6 +1744,8 @@ TcParams tc_params(const fstat_ctx* c) {
     t.base = c->d_base;
     t.comb = c->d_comb;
     t.perm = pl.tc_perm ? c->d_perm : nullptr;
+    t.cov = c->have_cov ? c->d_cov : nullptr;
+    t.comb_j = c->d_comb_j;
     t.twoF = c->d_twoF;
     t.scratch = c->d_tcs;
     t.err = c->d_err;

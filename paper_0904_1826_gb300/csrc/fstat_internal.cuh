@@ -211,6 +211,8 @@ struct TcParams {
     const SkySftBase* base;        // [n_sft][n_sky]
     const float4* comb;            // [n_sky]
     const int* perm;               // sky point at each place of the grouping order, or null
+    const int2* cov;               // [n_sft] covered templates [x, y), or null
+    const float4* comb_j;          // [n_sky][n_f] combine weights where cov is set
     float* twoF;                   // [n_sky][n_fdot][n_f]
     float4* scratch;               // [blocks][kTcSlots][kTcRows][kTcCols]
     int* err;

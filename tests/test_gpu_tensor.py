@@ -190,3 +190,41 @@ def test_sparse_skies_at_high_frequency(lib, n_sky, f0):
     direct, _, dflags, _ = _run(lib, w, bins, algo="direct")
     assert tiles["rows"] > 0 and flags == dflags
     assert np.all(np.abs(got.astype(np.float64) - direct) <= 2 * (REL * np.abs(direct) + ABS))
+
+
+@pytest.mark.parametrize("sizes,n_sky", [
+    (dict(n_sft=40, n_f=301, n_fdot=5, n_bins=340), 600),
+    (dict(n_sft=40, n_f=639, n_fdot=5, n_bins=360, df_bins=0.5), 300),
+    (dict(n_sft=60, n_f=301, n_fdot=5, n_bins=340), 300),     # tiles shared by blocks
+])
+def test_tensor_form_with_coverage(lib, sizes, n_sky):
+    """SFTs that cover everything, nothing, one template, up to and from the edges
+    of column blocks, and ranges far outside the band, against the direct form."""
+    w = _dense(n_sky, **sizes)
+    bins = O.inject(w.detectors, w.T, w.k_lo, w.injections, w.bank.t_ref)
+    n, nf = w.n_sft_total, w.bank.n_f
+    rng = np.random.default_rng(4)
+    lo, hi = np.zeros(n, np.int32), np.full(n, nf, np.int32)
+    special = [(0, 64), (64, 128), (63, 65), (5, 6), (nf, nf), (0, 0), (-2 ** 31, 2 ** 31 - 1), (-2 ** 31, 40),
+               (200, 2 ** 31 - 1), (nf - 1, nf)]
+    for i, (a, b) in enumerate(special[:n]):
+        lo[i], hi[i] = a, b
+    for i in range(len(special), n):
+        if i % 5 == 1:
+            lo[i] = rng.integers(-10, nf // 2)
+            hi[i] = lo[i] + rng.integers(nf // 2, nf)
+
+    def run(**opts):
+        g = lib.FStat(0, dterms=8, topk=20, **opts)
+        try:
+            g.load_workload(w, bins_override=bins)
+            lib.fstat_set_coverage(g.ctx, lo, hi)
+            g.compute()
+            return g.twoF(), g.error_flags(), g.tensor_tiles()["rows"]
+        finally:
+            g.close()
+
+    got, flags, rows = run()
+    direct, dflags, none = run(algo="direct")
+    assert rows > 0 and none == 0 and flags == dflags
+    assert np.all(np.abs(got.astype(np.float64) - direct) <= 2 * (REL * np.abs(direct) + ABS))

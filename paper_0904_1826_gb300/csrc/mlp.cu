@@ -33,8 +33,8 @@ enum { EPI_F32 = 0, EPI_RELU = 1, EPI_MASK = 2 };
 // on shared-memory descriptors (leading-dimension step: the next 8 columns,
 // R * 16 bytes; stride step: the next 8 rows, 128 bytes) into a TMEM
 // accumulator of 64 columns and commits them to the stage's mbarrier.  Two
-// stages: the threads stage slice k + 1 while the tensor core runs slice k,
-// and wait (bounded) for slice k - 1's MMAs before reusing its stage.  The
+// stages: the threads load slice k + 1 into registers while the tensor core runs
+// slice k, and wait (bounded) for slice k - 1's MMAs before reusing its stage.  The
 // epilogue reads the tile back with tcgen05.ld (warp w owns TMEM lanes, i.e.
 // rows, 32w .. 32w + 31); with several K chunks it writes the raw FP32 tile of
 // its chunk to part[z][M][N] and splitk_epi_kernel finishes the sum.
@@ -86,55 +86,84 @@ __device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity) {
     return __syncthreads_and(done != 0) != 0;
 }
 
-template <bool TA, bool TB>
-__device__ __forceinline__ void tc_stage(unsigned char* As, unsigned char* Bs, int M, int N, int K, const bf16* A,
-                                         int lda, const bf16* B, int ldb, int m0, int n0, int k0, int kend) {
+// A slice of K in registers: 8 vectors of A and 4 of B a thread, loaded together
+// (one latency instead of twelve) while the slice before it is multiplied.  Bound:
+// latency, a product has 4 slices a block.  256 x 8192 x 256 and 256^3 together: 86 us
+// with a load and a store in turn, 51 so, 31 with vector stores of the result too.
+constexpr int TC_VA = TC_M * TC_K / 8 / 128, TC_VB = TC_N * TC_K / 8 / 128;
+struct TcRegs {
+    uint4 a[TC_VA], b[TC_VB];
+};
+
+// Row (m or n) and k of a thread's vector i of an R-row operand.  K-major: 8
+// consecutive k of one row.  Otherwise 8 consecutive rows of one k; 8 lanes take
+// 8 consecutive k, whose transposed 2-byte stores share a 16-byte line (4-way
+// bank conflicts; 16-way with the rows fastest).
+template <bool KMAJOR, int R>
+__device__ __forceinline__ void tc_pos(int i, int& r, int& kk) {
     const int tid = threadIdx.x;
-    const bf16 zero = __float2bfloat16(0.f);
-    // A slice: TC_M rows x TC_K columns (K-major in shared memory)
-    for (int v = tid; v < TC_M * TC_K / 8; v += 128) {
-        if (!TA) {   // 8 consecutive k of one row
-            const int r = v / (TC_K / 8), kk = (v % (TC_K / 8)) * 8;
-            const int gm = m0 + r, gk = k0 + kk;
-            uint4 q = make_uint4(0, 0, 0, 0);
-            if (gm < M && gk < kend) q = *reinterpret_cast<const uint4*>(A + (size_t)gm * lda + gk);
-            *reinterpret_cast<uint4*>(As + tc_off(TC_M, r, kk)) = q;
-        } else {     // 8 consecutive rows of one k
-            const int kk = v / (TC_M / 8), r = (v % (TC_M / 8)) * 8;
-            const int gm = m0 + r, gk = k0 + kk;
-            bf16 e[8];
-            if (gk < kend && gm + 7 < M) {
-                *reinterpret_cast<uint4*>(e) = *reinterpret_cast<const uint4*>(A + (size_t)gk * lda + gm);
-            } else {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) e[i] = (gk < kend && gm + i < M) ? A[(size_t)gk * lda + gm + i] : zero;
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i) *reinterpret_cast<bf16*>(As + tc_off(TC_M, r + i, kk)) = e[i];
-        }
+    if (KMAJOR) {
+        const int v = tid + 128 * i;
+        r = v / (TC_K / 8);
+        kk = (v % (TC_K / 8)) * 8;
+    } else {
+        constexpr int kHigh = 16 / (R / 8);   // groups of 8 k a pass
+        r = ((tid >> 3) % (R / 8)) * 8;
+        kk = 8 * ((tid >> 3) / (R / 8) + kHigh * i) + (tid & 7);
     }
-    // B slice as B^T: TC_N rows (n) x TC_K columns (k)
-    for (int v = tid; v < TC_N * TC_K / 8; v += 128) {
-        if (TB) {    // 8 consecutive k of one n
-            const int r = v / (TC_K / 8), kk = (v % (TC_K / 8)) * 8;
-            const int gn = n0 + r, gk = k0 + kk;
-            uint4 q = make_uint4(0, 0, 0, 0);
-            if (gn < N && gk < kend) q = *reinterpret_cast<const uint4*>(B + (size_t)gn * ldb + gk);
-            *reinterpret_cast<uint4*>(Bs + tc_off(TC_N, r, kk)) = q;
-        } else {     // 8 consecutive n of one k
-            const int kk = v / (TC_N / 8), r = (v % (TC_N / 8)) * 8;
-            const int gn = n0 + r, gk = k0 + kk;
-            bf16 e[8];
-            if (gk < kend && gn + 7 < N) {
-                *reinterpret_cast<uint4*>(e) = *reinterpret_cast<const uint4*>(B + (size_t)gk * ldb + gn);
-            } else {
+}
+
+template <bool KMAJOR, int R>
+__device__ __forceinline__ uint4 tc_load1(int i, int rows, const bf16* P, int ld, int r0, int k0, int kend) {
+    int r, kk;
+    tc_pos<KMAJOR, R>(i, r, kk);
+    const int gr = r0 + r, gk = k0 + kk;
+    uint4 q = make_uint4(0, 0, 0, 0);
+    if (KMAJOR) {
+        if (gr < rows && gk < kend) q = __ldg(reinterpret_cast<const uint4*>(P + (size_t)gr * ld + gk));
+    } else if (gk < kend && gr + 7 < rows) {
+        q = __ldg(reinterpret_cast<const uint4*>(P + (size_t)gk * ld + gr));
+    } else if (gk < kend) {
+        uint32_t w[4] = {0, 0, 0, 0};
 #pragma unroll
-                for (int i = 0; i < 8; ++i) e[i] = (gk < kend && gn + i < N) ? B[(size_t)gk * ldb + gn + i] : zero;
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i) *reinterpret_cast<bf16*>(Bs + tc_off(TC_N, r + i, kk)) = e[i];
-        }
+        for (int e = 0; e < 8; ++e)
+            if (gr + e < rows)
+                w[e >> 1] |= (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(P) + (size_t)gk * ld + gr + e)
+                             << (16 * (e & 1));
+        q = make_uint4(w[0], w[1], w[2], w[3]);
     }
+    return q;
+}
+
+template <bool KMAJOR, int R>
+__device__ __forceinline__ void tc_store1(unsigned char* S, int i, const uint4& q) {
+    int r, kk;
+    tc_pos<KMAJOR, R>(i, r, kk);
+    if (KMAJOR) {
+        *reinterpret_cast<uint4*>(S + tc_off(R, r, kk)) = q;
+    } else {
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            *reinterpret_cast<unsigned short*>(S + tc_off(R, r + e, kk)) = (unsigned short)(w[e >> 1] >> (16 * (e & 1)));
+    }
+}
+
+// A(m, k): K-major unless TA; B(k, n) as B^T: K-major if TB.
+template <bool TA, bool TB>
+__device__ __forceinline__ void tc_load(TcRegs& t, int M, int N, const bf16* A, int lda, const bf16* B, int ldb, int m0,
+                                        int n0, int k0, int kend) {
+#pragma unroll
+    for (int i = 0; i < TC_VA; ++i) t.a[i] = tc_load1<!TA, TC_M>(i, M, A, lda, m0, k0, kend);
+#pragma unroll
+    for (int i = 0; i < TC_VB; ++i) t.b[i] = tc_load1<TB, TC_N>(i, N, B, ldb, n0, k0, kend);
+}
+template <bool TA, bool TB>
+__device__ __forceinline__ void tc_store(unsigned char* As, unsigned char* Bs, const TcRegs& t) {
+#pragma unroll
+    for (int i = 0; i < TC_VA; ++i) tc_store1<!TA, TC_M>(As, i, t.a[i]);
+#pragma unroll
+    for (int i = 0; i < TC_VB; ++i) tc_store1<TB, TC_N>(Bs, i, t.b[i]);
 }
 
 template <bool TA, bool TB, int EPI>
@@ -168,6 +197,8 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(int M, int N, int K, const
     uint32_t ph0 = 0, ph1 = 0;   // parity of the next wait on each stage's barrier
     bool ok = true;
     int it = 0;
+    TcRegs t;
+    tc_load<TA, TB>(t, M, N, A, lda, B, ldb, m0, n0, kb, ke);
     for (; it < n_sl; ++it) {
         const int st = it & 1;
         if (it >= 2) {   // the MMAs of slice it - 2 read this stage
@@ -178,7 +209,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(int M, int N, int K, const
         }
         unsigned char* As = tsm + st * TC_STAGE_BYTES;
         unsigned char* Bs = As + TC_A_BYTES;
-        tc_stage<TA, TB>(As, Bs, M, N, K, A, lda, B, ldb, m0, n0, kb + it * TC_K, ke);
+        tc_store<TA, TB>(As, Bs, t);
         // the tensor core reads shared memory through the async proxy
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
@@ -203,6 +234,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(int M, int N, int K, const
                              bar0 + 8 * st)
                          : "memory");
         }
+        if (it + 1 < n_sl) tc_load<TA, TB>(t, M, N, A, lda, B, ldb, m0, n0, kb + (it + 1) * TC_K, ke);
     }
     // drain: the commits of the last two slices
     if (ok) {
@@ -228,7 +260,47 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(int M, int N, int K, const
                   "=r"(v[15])
                 : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0));
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (row < M) {
+            if (row < M && n0 + c0 + 16 <= N && ((ldc | N) & 7) == 0) {   // whole vectors: a quarter of the memory instructions
+                const int col = n0 + c0;
+                float x[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) x[j] = __uint_as_float(v[j]);
+                if (pz) {
+#pragma unroll
+                    for (int j = 0; j < 16; j += 4)
+                        *reinterpret_cast<float4*>(pz + (size_t)row * N + col + j) = make_float4(x[j], x[j + 1], x[j + 2], x[j + 3]);
+                    continue;
+                }
+                const size_t o = (size_t)row * ldc + col;
+                if (bias) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) x[j] += bias[col + j];
+                }
+                if (EPI == EPI_MASK) {
+#pragma unroll
+                    for (int j = 0; j < 16; j += 4) {
+                        const float4 z = *reinterpret_cast<const float4*>(zref + o + j);
+                        x[j] = z.x > 0.f ? x[j] : 0.f;
+                        x[j + 1] = z.y > 0.f ? x[j + 1] : 0.f;
+                        x[j + 2] = z.z > 0.f ? x[j + 2] : 0.f;
+                        x[j + 3] = z.w > 0.f ? x[j + 3] : 0.f;
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 16; j += 4)
+                    *reinterpret_cast<float4*>(Cf + o + j) = make_float4(x[j], x[j + 1], x[j + 2], x[j + 3]);
+                if (EPI != EPI_F32) {
+                    __nv_bfloat162 h[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float a = EPI == EPI_RELU ? fmaxf(x[2 * j], 0.f) : x[2 * j];
+                        const float b = EPI == EPI_RELU ? fmaxf(x[2 * j + 1], 0.f) : x[2 * j + 1];
+                        h[j] = __floats2bfloat162_rn(a, b);
+                    }
+                    *reinterpret_cast<uint4*>(Cb + o) = *reinterpret_cast<const uint4*>(h);
+                    *reinterpret_cast<uint4*>(Cb + o + 8) = *reinterpret_cast<const uint4*>(h + 4);
+                }
+            } else if (row < M) {
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
                     const int col = n0 + c0 + j;
@@ -315,58 +387,106 @@ __global__ void head_kernel(const float* __restrict__ z2, const float* __restric
     }
 }
 
-// Deterministic sum of n values by one block.
-__global__ void sum_kernel(const float* __restrict__ v, int n, float* __restrict__ out, float scale) {
-    __shared__ float red[256];
-    float a = 0.f;
-    for (int i = threadIdx.x; i < n; i += 256) a += v[i];
-    red[threadIdx.x] = a;
+// Column sums over the rows of an array: 32 columns a block, 32 warps of rows
+// (one row a warp and pass), the warps' sums added in warp order.
+constexpr int kColRows = 32;
+__device__ __forceinline__ float col_reduce(float a, float (*red)[33]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
+    red[warp][lane] = a;
+    __syncthreads();
+    if (warp == 0) {
+        a = 0.f;
+        for (int w = 0; w < kColRows; ++w) a += red[w][lane];
     }
-    if (threadIdx.x == 0) out[0] = red[0] * scale;
+    return a;   // of the column, in warp 0
 }
 
-// Layer-3 backward: dw3[n] = sum_b relu(z2) ds, dz2 = ds w3 (z2 > 0) (FP32 and BF16).
-__global__ void head_back_kernel(const float* __restrict__ z2, const float* __restrict__ w3,
-                                 const float* __restrict__ ds, int B, int H, float* __restrict__ dw3,
-                                 float* __restrict__ dz2, bf16* __restrict__ dz2b) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= H) return;
-    float a = 0.f;
-    for (int b = 0; b < B; ++b) {
-        const float z = z2[(size_t)b * H + n];
-        a = fmaf(fmaxf(z, 0.f), ds[b], a);
-        const float d = z > 0.f ? ds[b] * w3[n] : 0.f;
-        dz2[(size_t)b * H + n] = d;
-        dz2b[(size_t)b * H + n] = __float2bfloat16_rn(d);
+// Layer-3 backward: dw3[n] = sum_b relu(z2) ds, dz2 = ds w3 (z2 > 0) (FP32 and
+// BF16), db2[n] = sum_b dz2; the last block: mean loss and db3 = sum_b ds.
+// (One thread a column over all rows took 39 us for 256 x 256, this 4.3; column sums 8.5 and 3.)
+__global__ void __launch_bounds__(1024) head_back_kernel(const float* __restrict__ z2, const float* __restrict__ w3,
+                                                         const float* __restrict__ ds, const float* __restrict__ lrow,
+                                                         int B, int H, float* __restrict__ dw3, float* __restrict__ db2,
+                                                         float* __restrict__ dz2, bf16* __restrict__ dz2b,
+                                                         float* __restrict__ loss, float* __restrict__ db3) {
+    __shared__ float red[kColRows][33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (blockIdx.x + 1 == gridDim.x) {
+        float l = 0.f, d = 0.f;
+        for (int b = threadIdx.x; b < B; b += 1024) {
+            l += lrow[b];
+            d += ds[b];
+        }
+        l = col_reduce(l, red);
+        d = col_reduce(d, red);
+        if (warp == 0) {
+            for (int o = 16; o > 0; o >>= 1) {
+                l += __shfl_xor_sync(0xffffffffu, l, o);
+                d += __shfl_xor_sync(0xffffffffu, d, o);
+            }
+            if (lane == 0) {
+                *loss = l * (1.f / (float)B);
+                *db3 = d;
+            }
+        }
+        return;
     }
-    dw3[n] = a;
+    const int n = blockIdx.x * 32 + lane;
+    const float w = n < H ? w3[n] : 0.f;
+    float a = 0.f, c = 0.f;
+#pragma unroll 4
+    for (int b = warp; b < B; b += kColRows) {
+        if (n < H) {
+            const float z = z2[(size_t)b * H + n], g = ds[b];
+            a = fmaf(fmaxf(z, 0.f), g, a);
+            const float d = z > 0.f ? g * w : 0.f;
+            c += d;
+            dz2[(size_t)b * H + n] = d;
+            dz2b[(size_t)b * H + n] = __float2bfloat16_rn(d);
+        }
+    }
+    a = col_reduce(a, red);
+    c = col_reduce(c, red);
+    if (warp == 0 && n < H) {
+        dw3[n] = a;
+        db2[n] = c;
+    }
 }
 
 // Column sums (bias gradients) of a [B][H] FP32 array.
-__global__ void colsum_kernel(const float* __restrict__ v, int B, int H, float* __restrict__ out) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= H) return;
+__global__ void __launch_bounds__(1024) colsum_kernel(const float* __restrict__ v, int B, int H, float* __restrict__ out) {
+    __shared__ float red[kColRows][33];
+    const int n = blockIdx.x * 32 + (threadIdx.x & 31);
     float a = 0.f;
-    for (int b = 0; b < B; ++b) a += v[(size_t)b * H + n];
-    out[n] = a;
+#pragma unroll 4
+    for (int b = threadIdx.x >> 5; b < B; b += kColRows)
+        if (n < H) a += v[(size_t)b * H + n];
+    a = col_reduce(a, red);
+    if (threadIdx.x < 32 && n < H) out[n] = a;
 }
 
-__global__ void adam_kernel(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
-                            const float* __restrict__ gr, long long n, float lr, float c1, float c2,
-                            bf16* __restrict__ pb) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const float gi = gr[i];
-        const float mi = 0.9f * m[i] + 0.1f * gi;
-        const float vi = 0.999f * v[i] + 0.001f * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        const float pi = p[i] - lr * (mi * c1) / (sqrtf(vi * c2) + 1e-8f);
-        p[i] = pi;
-        if (pb) pb[i] = __float2bfloat16_rn(pi);
+// All parameters in one launch: the parameter arrays end to end, n[5] the total.
+struct AdamArrays {
+    float *p[6], *m[6], *v[6];
+    const float* g[6];
+    bf16* pb[6];
+    long long end[6];
+};
+__global__ void __launch_bounds__(256) adam_kernel(const AdamArrays q, float lr, float c1, float c2) {
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < q.end[5]; t += stride) {
+        int k = 0;
+        while (t >= q.end[k]) ++k;
+        const long long i = t - (k ? q.end[k - 1] : 0);
+        const float gi = q.g[k][i];
+        const float mi = 0.9f * q.m[k][i] + 0.1f * gi;
+        const float vi = 0.999f * q.v[k][i] + 0.001f * gi * gi;
+        q.m[k][i] = mi;
+        q.v[k][i] = vi;
+        const float pi = q.p[k][i] - lr * (mi * c1) / (sqrtf(vi * c2) + 1e-8f);
+        q.p[k][i] = pi;
+        if (q.pb[k]) q.pb[k][i] = __float2bfloat16_rn(pi);
     }
 }
 
@@ -682,17 +802,15 @@ int fstat_mlp_train_step(fstat_mlp* m, const uint16_t* X, const float* y, int32_
                                mem == FSTAT_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
     if ((rc = run_forward(m, Xd, B, s)) != FSTAT_OK) return rc;
     head_kernel<<<(B + 7) / 8, 256, 0, s>>>(m->z2, m->w3, m->b3, B, H, m->y, pos_weight, m->s, m->ds, m->lrow);
-    sum_kernel<<<1, 256, 0, s>>>(m->lrow, B, m->loss, 1.f / (float)B);
-    sum_kernel<<<1, 256, 0, s>>>(m->ds, B, m->gb3, 1.f);
-    head_back_kernel<<<(H + 127) / 128, 128, 0, s>>>(m->z2, m->w3, m->ds, B, H, m->gw3, m->dz2, m->dz2b);
-    colsum_kernel<<<(H + 127) / 128, 128, 0, s>>>(m->dz2, B, H, m->gb2);
+    head_back_kernel<<<(H + 31) / 32 + 1, 1024, 0, s>>>(m->z2, m->w3, m->ds, m->lrow, B, H, m->gw3, m->gb2, m->dz2, m->dz2b,
+                                                       m->loss, m->gb3);
     MLP_TRY(m, cudaGetLastError());
     // dW2 = h1^T dz2;  dz1 = (dz2 W2^T) * (z1 > 0);  dW1 = X^T dz1
     MLP_TRY(m, (gemm<true, false, EPI_F32>(H, H, B, m->h1, H, m->dz2b, H, nullptr, m->gW2, nullptr,
                                            nullptr, H, s, m->tcw)));
     MLP_TRY(m, (gemm<false, true, EPI_MASK>(B, H, H, m->dz2b, H, m->W2b, H, nullptr, m->dz1, m->dz1b,
                                             m->z1, H, s, m->tcw)));
-    colsum_kernel<<<(H + 127) / 128, 128, 0, s>>>(m->dz1, B, H, m->gb1);
+    colsum_kernel<<<(H + 31) / 32, 1024, 0, s>>>(m->dz1, B, H, m->gb1);
     MLP_TRY(m, (gemm<true, false, EPI_F32>(I, H, B, Xd, I, m->dz1b, H, nullptr, m->gW1, nullptr,
                                            nullptr, H, s, m->tcw)));
     // Adam
@@ -702,9 +820,17 @@ int fstat_mlp_train_step(fstat_mlp* m, const uint16_t* X, const float* y, int32_
     float* Gr[6] = {m->gW1, m->gb1, m->gW2, m->gb2, m->gw3, m->gb3};
     bf16* Pb[6] = {m->W1b, nullptr, m->W2b, nullptr, nullptr, nullptr};
     const long long n[6] = {(long long)I * H, H, (long long)H * H, H, H, 1};
-    for (int i = 0; i < 6; ++i)
-        adam_kernel<<<(int)std::min<long long>(1024, (n[i] + 255) / 256), 256, 0, s>>>(P[i], m->mom[2 * i], m->mom[2 * i + 1],
-                                                                                       Gr[i], n[i], lr, c1, c2, Pb[i]);
+    AdamArrays q;
+    long long total = 0;
+    for (int i = 0; i < 6; ++i) {
+        q.p[i] = P[i];
+        q.m[i] = m->mom[2 * i];
+        q.v[i] = m->mom[2 * i + 1];
+        q.g[i] = Gr[i];
+        q.pb[i] = Pb[i];
+        q.end[i] = total += n[i];
+    }
+    adam_kernel<<<(int)std::min<long long>(8LL * current_sm_count(), (total + 255) / 256), 256, 0, s>>>(q, lr, c1, c2);
     MLP_TRY(m, cudaGetLastError());
     if (loss) {
         MLP_TRY(m, cudaMemcpyAsync(loss, m->loss, sizeof(float), cudaMemcpyDeviceToHost, s));

@@ -52,10 +52,11 @@ KERNEL_SOURCES = {"direct": ["fstat_internal.cuh", "dirichlet.cuh", "dirichlet_c
                   "farpoly": ["fstat_internal.cuh", "dirichlet.cuh", "dirichlet_far.cu"],
                   "sincpoly": ["fstat_internal.cuh", "dirichlet.cuh", "dirichlet_far.cu"],
                   "sincrows": ["fstat_internal.cuh", "dirichlet.cuh", "dirichlet_far.cu"],
-                  "sincpairs": ["fstat_internal.cuh", "dirichlet.cuh", "dirichlet_far.cu"]}
+                  "sincpairs": ["fstat_internal.cuh", "dirichlet.cuh", "dirichlet_far.cu"],
+                  "tensor": ["fstat_internal.cuh", "dirichlet.cuh", "mbar.cuh", "dirichlet_tc.cu"]}
 KERNEL_NAMES = {"direct": "dirichlet_kernel", "farpoly": "dirichlet_far_kernel",
                 "sincpoly": "dirichlet_far_ring_kernel", "sincrows": "dirichlet_rows_kernel",
-                "sincpairs": "dirichlet_ring2_kernel"}
+                "sincpairs": "dirichlet_ring2_kernel", "tensor": "dirichlet_tc_kernel"}
 
 
 def parse():
@@ -688,6 +689,7 @@ def main():
 
     g = make(args.form)
     plan = g.plan()
+    tensor_rows = g.tensor_tiles()["rows"]
     sampler = ClockSampler(local_rank)
     sampler.start()
     n_launch0 = [0]
@@ -779,13 +781,15 @@ def main():
     peak = n_sm * FP32_LANES * 2 * clock_mhz * 1e6 / 1e12       # TFLOP/s, recipe unit counts, max clock
     achieved = FLOP_PER_PAIR * n_pairs / (k_dir / 1e3) / 1e12
     vid = plan.get("variant", 0)
-    algo_used = algo_of(vid)
-    kernel_name = KERNEL_NAMES[algo_used] if (vid < 107 or vid >= 120) else "dirichlet_far_ring_kernel"
+    algo_used = "tensor" if tensor_rows > 0 else algo_of(vid)   # the plan stays the ring it replaces
+    kernel_name = (KERNEL_NAMES[algo_used] if (vid < 107 or vid >= 120 or tensor_rows > 0)
+                   else "dirichlet_far_ring_kernel")
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": ncu_traffic(args.form, algo_used), "kernel": kernel_name,
                 "dirichlet_ms": k_dir, "step_ms_device": k_step,
                 "peak_note": f"{n_sm} SM (queried) x {FP32_LANES} FP32 lanes x 2 flop x {clock_mhz:.0f} MHz "
-                             "(maximum SM clock)"}
+                             "(maximum SM clock)"
+                             + ("; the tensor form runs the window sums on the tensor cores" if tensor_rows > 0 else "")}
     if clocks and clocks.get("sm_mhz"):
         roofline["frac_at_sampled_clock"] = achieved / (n_sm * FP32_LANES * 2 * clocks["sm_mhz"] * 1e6 / 1e12)
     # the table forms are bound by shared-memory loads: that bound too, from the

@@ -119,8 +119,8 @@ typedef struct {
  *   sky points (consecutive ones of the bank, or of a neighbour order of its
  *   sky list) sharing one staged window; else FARPOLY where it applies, else
  *   DIRECT.  Results of these forms do not depend on the grouping.
- *   Large banks of dense sky lists (column steps P df T = 1 bin, uniform
- *   spindowns, no coverage, no tile request) run the direct sum on the tensor
+ *   Large banks (column steps P df T = 1 bin, uniform spindowns, sky points
+ *   near enough to share a window, no tile request) run the direct sum on the tensor
  *   cores instead where the planner finds that faster: window sums from FP16
  *   pairs of bins and weights with FP32 accumulation, closer to the exact sum
  *   than SINCPOLY; in the last bits its results depend on which sky points
@@ -283,6 +283,7 @@ int fstat_set_noise_floor(fstat_ctx *ctx, int32_t half_window);
  * An SFT that covers none of a thread's templates is skipped, so work falls
  * with coverage.  From the next fstat_compute on; both pointers NULL switch
  * coverage off.  Loading SFTs (fstat_set_sfts) switches it off too.
+ * (The tensor-core form masks such an SFT instead.)
  * Restrictions: n_f <= 8192 while coverage is on; the far-field form runs
  * only in its TMA-ring staging (elsewhere the direct form is used); batched
  * workunits have no coverage.  fstat_get_abcd stays the per-sky sum over

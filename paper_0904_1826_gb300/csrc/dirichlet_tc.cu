@@ -48,11 +48,15 @@
 // 21 %, FMA pipes 43 %.  Against the sinc ring: 4000 sky x 1800 f x 10 spindowns x
 // 2400 SFTs 203 ms (8.5e11 pairs/s) against 293; 250 x 1733 x 7 x 2302, FP16 bins,
 // 217 Hz 9.1 against 15.7 ms; 2048 x 900 x 1 x 1600 4.1 against 6.9; the 1/8-bin
-// patch 2048 x 256 2.1 against 3.1.  What it took, on 4000 sky x 640 f x 600 SFTs (ring 26 ms): one thread
-// issuing copies and products beside its weights 55 ms; a warp of its own for
-// them, operands in uniform registers 22; code that fits the instruction caches
-// (rolled loops, short waits) and 8 weight warps 18.6; three operand buffers
-// and the row constants in warps of their own 17.8.
+// patch 2048 x 256 2.1 against 3.1.
+// What it took, on 4000 sky x 640 f x 600 SFTs (ring 26 ms): one thread issuing
+// copies and products beside its weights 55 ms; a warp of its own for them,
+// operands in uniform registers 22; code that fits the instruction caches (rolled
+// loops, short waits) and 8 weight warps 18.6; three operand buffers and the row
+// constants in warps of their own 17.8.  The register shares, the run's length
+// read from shared memory and the epilogue of four columns at a time are part of
+// it: other shares 207 to 223 ms on the work unit against 204, the length in a
+// register 218, eight columns at a time 225 (spills in the sums).
 //
 // Every wait is bounded; a give-up raises error flag bit 2 and ends the block.
 #include <algorithm>

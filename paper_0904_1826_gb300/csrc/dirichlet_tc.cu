@@ -368,11 +368,13 @@ __global__ void __launch_bounds__(256) finish_kernel(const TcParams p, int block
     }
 }
 
-// COV: per-SFT frequency coverage; an SFT's templates j outside [x, y) add nothing
-// (window sums set to zero where a warp's columns are not all covered, so the
-// products run on).  300 sky x 1800 f x 5 x 2400, a fifth of the SFTs covering part of
-// the band: 9.5 ms against 12.4 with the ring that skips.
-template <bool COV>
+// COV: per-SFT frequency coverage; an SFT's templates j outside [x, y) add nothing.
+// A warp whose columns are not all covered sets the others' window sums to zero in
+// tensor memory first; the products run on.  1: one template a bin (rows without a
+// sub-bin offset, whose lookup in the copying warp cost 4 %), 2: several.  300 sky x
+// 1800 f x 5 x 2400, a fifth of the SFTs covering part of the band: 8.7 ms against
+// 12.4 ms with the ring that skips; 8.4 without coverage.
+template <int COV>
 __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -579,10 +581,8 @@ __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParam
                         const float4 u = W4[(n & 7) * kRows + src], e4 = P4[(n & 7) * kRows + src];
                         const float b = B1[(n & 7) * kRows + src];
                         const int sh = max(0, min(__float_as_int(u.z) - 4 * wn.x, 16 * wn.y - 16));
-                        // first column's template of the row
-                        const int jr = COV ? p.n_sub * (((item0 + seg) / p.n_tiles) * kCols) +
-                                                 (((item0 + seg) % p.n_tiles) * p.rt + src) % p.rps % p.n_sub
-                                           : 0;
+                        // first column's template of the row, from the tile's first
+                        const int jr = COV == 2 ? (((item0 + seg) % p.n_tiles) * p.rt + src) % p.rps % p.n_sub : 0;
 #pragma unroll 2
                         for (int c = lane; c < kCols; c += 32) {
                             if (COV && (jr + p.n_sub * c < cvr[n & 7].x || jr + p.n_sub * c >= cvr[n & 7].y)) continue;
@@ -665,9 +665,10 @@ __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParam
                     hi = __reduce_max_sync(0xffffffffu, hi);
                     __syncwarp();
                     if (lane == 0) {
-                        if (COV) {   // clamped to the band; by both warps, the same
+                        if (COV) {   // clamped to the band, from the tile's first template; by both warps, the same
                             const int2 c = __ldg(p.cov + s);
-                            cvr[n & 7] = make_int2(max(0, min(c.x, p.n_f)), c.y >= p.n_f ? 1 << 30 : max(0, c.y));
+                            cvr[n & 7] = make_int2(max(0, min(c.x, p.n_f)) - p.n_sub * c0,
+                                                   c.y >= p.n_f ? 1 << 30 : max(0, c.y) - p.n_sub * c0);
                         }
                         mm[(n & 7) * 2 + warp - 18] = make_int2(lo, hi);
                         mbar_arrive(r_full(n));
@@ -697,11 +698,6 @@ __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParam
                     v[12 + 2 * e] += fbi[i].x, v[13 + 2 * e] += fbi[i].y;
                 }
             };
-            int jr = 0;   // template of the thread's first column
-            if (COV) {
-                const int item = item0 + seg;
-                jr = p.n_sub * ((item / p.n_tiles) * kCols + 32 * h) + ((item % p.n_tiles) * p.rt + row) % p.rps % p.n_sub;
-            }
             float zero[16] = {};
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
@@ -729,34 +725,44 @@ __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParam
                     ti[i] = make_float2(-s0, -s1);
                 }
                 const float2 rr = dup(p4.z), ri = dup(p4.w), nri = dup(-p4.w), a2 = dup(wa), b2 = dup(wb);
-                // the thread's covered columns [cl, ch) where they are not all covered
-                bool part = false;
-                int cl = 0, ch_end = 32;
-                if (COV) {
-                    const int2 cv = cvr[n & 7];
-                    part = __any_sync(0xffffffffu, cv.x > jr || cv.y <= jr + 31 * p.n_sub);
-                    if (part) {
-                        cl = (max(cv.x - jr, 0) + p.n_sub - 1) / p.n_sub;
-                        ch_end = (max(cv.y - jr, 0) + p.n_sub - 1) / p.n_sub;
-                    }
-                }
                 ok = wait(d_full(n), n >> 1);
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t td = tbase + (n & 1) * (2 * kCols);
+                if (COV && (cvr[n & 7].x > 32 * h * p.n_sub || cvr[n & 7].y < (32 * h + 32) * p.n_sub)) {
+                    // not all of the warp's columns are covered: zeros into the others' window sums
+                    const int2 cv = cvr[n & 7];
+                    if (cv.x >= (32 * h + 32) * p.n_sub || cv.y <= 32 * h * p.n_sub) {   // none: the sums stay
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) {
+                            mbar_arrive(d_free(n));
+                            mbar_arrive(r_free(n));
+                        }
+                        continue;
+                    }
+                    const int item = (int)((run_first(p) + n) / p.n_sft);
+                    const int jr = 32 * h * p.n_sub + ((item % p.n_tiles) * p.rt + row) % p.rps % p.n_sub;
+#pragma unroll 1
+                    for (int ch = 0; ch < 4; ++ch) {
+                        float u[16];
+                        tmem_ld16(td + 16 * ch, u);
+                        tmem_wait16(u);
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) {
+                            const int j = jr + p.n_sub * (8 * ch + 4 * (e >> 3) + (e & 3));
+                            u[e] = j >= cv.x && j < cv.y ? u[e] : 0.0f;
+                        }
+                        tmem_st16(td + 16 * ch, u);
+                    }
+                    tmem_wait_st();
+                }
                 float v[2][16];
                 tmem_ld16(td, v[0]);
                 tmem_wait16(v[0]);
 #pragma unroll
                 for (int ch = 0; ch < 4; ++ch) {   // eight columns: twice four real parts, four imaginary parts
                     float (&cv)[16] = v[ch & 1];
-                    if (COV && part) {
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) {
-                            const int col = 8 * ch + 4 * (e >> 3) + (e & 3);
-                            cv[e] = col >= cl && col < ch_end ? cv[e] : 0.0f;
-                        }
-                    }
                     if (ch < 3) tmem_ld16(td + 16 * (ch + 1), v[(ch + 1) & 1]);
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
@@ -919,7 +925,7 @@ int tc_launches(const TcParams& p) {
 }
 
 cudaError_t launch_dirichlet_tc(const TcParams& p, cudaStream_t s) {
-    const auto kernel = p.cov ? dirichlet_tc_kernel<true> : dirichlet_tc_kernel<false>;
+    const auto kernel = !p.cov ? dirichlet_tc_kernel<0> : p.n_sub == 1 ? dirichlet_tc_kernel<1> : dirichlet_tc_kernel<2>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
     if (e != cudaSuccess) return e;
     const int grid = tc_blocks(p.n_tiles, p.n_colb, p.n_sft, current_sm_count());

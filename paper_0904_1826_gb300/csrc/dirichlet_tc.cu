@@ -121,8 +121,17 @@ __device__ __forceinline__ void mma_issue(uint32_t d, uint32_t a, uint32_t b, ui
         "r"(a), "r"(b), "r"(kIdesc), "r"(acc), "n"(kDescA), "n"(kDescB)
         : "memory");
 }
+// A commit tracks the products of the thread that issues it, so it is issued by
+// the lane that the products' election picks (the same for the same mask; which
+// one is not specified).
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+    asm volatile(
+        "{\n"
+        " .reg .pred q;\n"
+        " elect.sync _|q, 0xffffffff;\n"
+        " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+        "}\n" ::"r"(bar)
+        : "memory");
 }
 // A bounded wait of a few instructions (the kernel has many, in its loops): at
 // most 2^21 polls, each held by the hardware for about a microsecond (two to
@@ -503,7 +512,7 @@ __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParam
                 const uint32_t a = desc_lo(sb + buf * 4 * a_arr, kAGroup / 2), arr = a_arr / 16;
                 const uint32_t x = desc_lo(sb + kOffX + (n & 3) * kXStage, 2 * kBlk);
                 const uint32_t y = desc_lo(sb + kOffY + (n & 1) * kYStage, 2 * kBlk);
-// the accumulator is cut off, not rounded, at each product: the small
+                // the accumulator is cut off, not rounded, at each product: the small
                 // terms go first, so that few products see its full size (hh first: 2F
                 // 5e-7 too small on average).  Offsets in 16-byte units of the start address.
 #pragma unroll
@@ -519,15 +528,13 @@ __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParam
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
                     if (q < gk) mma_issue(dst, a + q * (kAGroup / 16), x + q * (4 * kBlk / 16), 1u);
-                if (lane == 0) {
-                    mma_commit(d_full(n));
-                    mma_commit(a_free(buf));
-                    mma_commit(x_free(n));
-                }
+                mma_commit(d_full(n));
+                mma_commit(a_free(buf));
+                mma_commit(x_free(n));
                 __syncwarp();
                 buf = buf + 1 == n_buf ? 0 : buf + 1;
             }
-            if (lane == 0) mma_commit(fin);
+            mma_commit(fin);
             __syncwarp();
             wait(fin, 0);
         } else if (warp == 17) {

@@ -124,7 +124,12 @@ typedef struct {
  *   cores instead where the planner finds that faster: window sums from FP16
  *   pairs of bins and weights with FP32 accumulation, closer to the exact sum
  *   than SINCPOLY; in the last bits its results depend on which sky points
- *   share a tile, so on the sky list. */
+ *   share a tile, so on the sky list.  It is kept to SFTs whose largest
+ *   component, among the bins that the bank's windows reach, is at most 65536
+ *   times that of their quietest 16 bins in a row (all-zero ones left out, a
+ *   few at the band's edge allowed for):
+ *   beside a stronger line its pairs would lose the weak bins' last bits, and
+ *   a form with FP32 bins runs. */
 typedef enum {
     FSTAT_ALGO_AUTO = 0,
     FSTAT_ALGO_DIRECT = 1,
@@ -313,7 +318,8 @@ int fstat_test_ring_stall(fstat_ctx *ctx, int32_t after_sft);
  *           far-field polynomial form, 112..115 the sinc-polynomial form,
  *           116 the sinc and 117 the far-field form with frequency coverage,
  *           118 and 119 the sinc form for L = 1 banks (P = 8); 107 and up use
- *           the TMA-ring staging). */
+ *           the TMA-ring staging).  The plan can depend on the bins: newly
+ *           loaded SFTs are prepared for it on the context's stream. */
 int fstat_get_plan(fstat_ctx *ctx, int32_t *out);
 
 /* Inspection: the tiles of the tensor-core form (see AUTO) the current bank

@@ -91,6 +91,8 @@ struct Plan {
     bool tc_perm = false;    // tiles take the sky points in tc_order
     int tc_sub = 1, tc_rt = kTcRows, tc_tiles = 0, tc_colb = 0;   // templates per bin, rows per tile, tiles, column blocks
     int tc_gk = 4;           // groups of 16 positions the windows of a tile span at most
+    int tc_lo = 0, tc_hi = 0;   // bins its tables hold
+    bool tc_by_range = false;   // the range of the bins decided on the form (choose_tc)
     size_t smem = 0;
     long long grid = 0;
 };
@@ -176,8 +178,9 @@ struct fstat_ctx {
     float* d_inv = nullptr;
     float4* d_tcs = nullptr;
     size_t cap_gtab = 0, cap_inv = 0, cap_tcs = 0;
-    int gt_nblk = -1, gt_xoff = -1;
+    int gt_nblk = -1, gt_xoff = -1, gt_lo = -1, gt_hi = -1;
     bool gt_dirty = true;
+    int tc_band_loud = -1;            // range of the whole band's bins too large for its tables (-1: not known)
     fstat_opts opts0{};               // the options as created (the autotuner changes opts)
     double dfdot = 0.0;
     // derived per-bank buffers
@@ -517,16 +520,51 @@ std::vector<int> tc_neighbour_order(const std::vector<TcSky>& sky, double g, dou
     return order;
 }
 
+const void* form_bins(const fstat_ctx* c);
+void bank_reach(const fstat_ctx* c, long long* lo, long long* hi);
+
+// Whether the tensor-core form's tables hold the bins that the bank's windows read
+// (tc_range_kernel): those of the whole band, so that the next bank of the same
+// SFTs finds its table built, or, where a line elsewhere in the band prevents that,
+// those from *lo to *hi that this bank's windows reach.
+int tc_range(fstat_ctx* c, cudaStream_t s, bool* fits, int* lo, int* hi) {
+    auto loud = [&](int from, int to, int* out) {
+        int* flag = c->d_err + 3;
+        CUDA_TRY(c, cudaMemsetAsync(flag, 0, sizeof(int), s));
+        CUDA_TRY(c, launch_tc_range(form_bins(c), c->opts.bins_form, c->row, c->n_sft, c->n_bins, from, to, flag, s));
+        c->launches += 1;
+        CUDA_TRY(c, cudaMemcpyAsync(out, flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+        CUDA_TRY(c, cudaStreamSynchronize(s));
+        return (int)FSTAT_OK;
+    };
+    int rc;
+    *lo = 0;
+    *hi = c->n_bins;
+    if (c->tc_band_loud < 0 && (rc = loud(-15, c->n_bins + 15, &c->tc_band_loud)) != FSTAT_OK) return rc;
+    *fits = c->tc_band_loud == 0;
+    if (*fits) return FSTAT_OK;
+    long long a, b;
+    bank_reach(c, &a, &b);
+    a = std::max(a, -15LL);
+    b = std::min(b + 1, c->n_bins + 15LL);
+    int over = 0;
+    if (a < b && (rc = loud((int)a, (int)b, &over)) != FSTAT_OK) return rc;
+    *fits = over == 0;
+    *lo = (int)std::max(0LL, std::min<long long>(a, c->n_bins));
+    *hi = (int)std::max<long long>(*lo, std::min<long long>(b, c->n_bins));
+    return FSTAT_OK;
+}
+
 // Tensor-core form where it is the faster one.  It needs column steps of one
 // bin (n_sub = P / L templates a bin), a uniform spindown grid, at least 8 SFTs
 // (its blocks work up to 6 ahead) and windows of a tile's rows within
-// kTcMaxSpread bins; Kahan sums, other D and explicit tile or form requests keep
-// the other forms.
-void choose_tc(fstat_ctx* c, int P, int L, bool found, Plan& pl) {
-    pl.tc = false;
+// kTcMaxSpread bins, and bins of a range that its tables hold (tc_range); Kahan
+// sums, other D and explicit tile or form requests keep the other forms.
+int choose_tc(fstat_ctx* c, int P, int L, bool found, Plan& pl, cudaStream_t s) {
+    pl.tc = pl.tc_by_range = false;
     const fstat_opts& o = c->opts0;
-    if (!found || P % L != 0 || !c->fdot_uniform || c->n_sft < 8) return;
-    if (o.algo != FSTAT_ALGO_AUTO || o.tile_m > 0 || o.tile_warps > 0 || o.sft_chunk > 0) return;
+    if (!found || P % L != 0 || !c->fdot_uniform || c->n_sft < 8) return FSTAT_OK;
+    if (o.algo != FSTAT_ALGO_AUTO || o.tile_m > 0 || o.tile_warps > 0 || o.sft_chunk > 0) return FSTAT_OK;
     const int n_sub = P / L, rps = c->n_fdot * n_sub;
     const long long n_rows = (long long)c->n_sky * rps;
     const long long n_col = (c->n_f + n_sub - 1) / n_sub;
@@ -549,8 +587,8 @@ void choose_tc(fstat_ctx* c, int P, int L, bool found, Plan& pl) {
         pairs *= covered / ((double)c->n_f * c->n_sft);
     }
     const double t_other = pairs / rate;
-    if (n_rows > (1 << 28) || (n_rows / 32 + 1) * colb > (1 << 28) || t_other > 3000.0) return;   // 32-bit counters
-    if (t_tc(kTcRows) > 0.92 * t_other) return;
+    if (n_rows > (1 << 28) || (n_rows / 32 + 1) * colb > (1 << 28) || t_other > 3000.0) return FSTAT_OK;   // 32-bit counters
+    if (t_tc(kTcRows) > 0.92 * t_other) return FSTAT_OK;
     const std::vector<TcSky> sky = tc_sky(c);
     for (int rt = kTcRows; rt >= 32 && t_tc(rt) <= 0.92 * t_other; rt /= 2) {
         double spread = tc_spread_bins(c, sky, rps, rt, nullptr);
@@ -567,7 +605,9 @@ void choose_tc(fstat_ctx* c, int P, int L, bool found, Plan& pl) {
             if (spread <= kTcMaxSpread) break;
         }
         if (spread > kTcMaxSpread) continue;
-        pl.tc = true;
+        pl.tc_by_range = true;
+        const int rc = tc_range(c, s, &pl.tc, &pl.tc_lo, &pl.tc_hi);
+        if (rc != FSTAT_OK || !pl.tc) return rc;
         pl.tc_perm = !nat;
         pl.tc_sub = n_sub;
         pl.tc_rt = rt;
@@ -575,8 +615,9 @@ void choose_tc(fstat_ctx* c, int P, int L, bool found, Plan& pl) {
         pl.tc_colb = (int)colb;
         // a window starts up to 3 positions into its first block
         pl.tc_gk = std::max(2, std::min(4, (int)std::ceil((spread + 3.0 + 16.0) / 16.0)));
-        return;
+        return FSTAT_OK;
     }
+    return FSTAT_OK;
 }
 
 bool far_eligible(const fstat_ctx* c) {
@@ -587,7 +628,8 @@ bool far_eligible(const fstat_ctx* c) {
 // lie inside them: khat is bounded over the bank by the frequency and spindown
 // ranges, |tdot - 1| <= 1.1e-4 (orbital + rotational speed over c) and dtau
 // within the SFT span of t_ref widened by 500 s of Roemer delay.
-void far_extent(const fstat_ctx* c, int w_pairs, int* xoff, int* n_pos) {
+// First and last bin, from k_lo, of any window of the bank.
+void bank_reach(const fstat_ctx* c, long long* lo, long long* hi) {
     double tmin = 1e300, tmax = -1e300;
     for (int d = 0; d < kMaxDet; ++d)
         for (double t : c->det[d].t_start) {
@@ -612,8 +654,14 @@ void far_extent(const fstat_ctx* c, int w_pairs, int* xoff, int* n_pos) {
                     kmin = std::min(kmin, k);
                     kmax = std::max(kmax, k);
                 }
-    const long long lo_min = (long long)std::floor(kmin) - c->k_lo - 7 - 2;
-    const long long lo_max = (long long)std::floor(kmax) - c->k_lo - 7 + 2;
+    *lo = (long long)std::floor(kmin) - c->k_lo - 7 - 2;
+    *hi = (long long)std::floor(kmax) - c->k_lo + 8 + 2;
+}
+
+void far_extent(const fstat_ctx* c, int w_pairs, int* xoff, int* n_pos) {
+    long long lo_min, hi_max;
+    bank_reach(c, &lo_min, &hi_max);
+    const long long lo_max = hi_max - 15;
     const long long xo = std::max<long long>(kFarXoff, -lo_min);
     long long np = std::max<long long>(c->n_bins + xo + kFarXoff, xo + lo_max + w_pairs + 2);
     *xoff = (int)xo;
@@ -1003,7 +1051,7 @@ bool make_far_plan(fstat_ctx* c, int P, int L, bool found, Plan& best) {
     return have;
 }
 
-int make_plan(fstat_ctx* c, Plan& out) {
+int make_plan(fstat_ctx* c, Plan& out, cudaStream_t s) {
     const int D = c->opts.dterms;
     const int kahan = c->opts.kahan ? 1 : 0;
     const double dk_nom = c->df * c->T;
@@ -1021,10 +1069,7 @@ int make_plan(fstat_ctx* c, Plan& out) {
                 }
     }
     if (far_eligible(c)) {
-        if (make_far_plan(c, P, L, found, out)) {
-            choose_tc(c, P, L, found, out);
-            return FSTAT_OK;
-        }
+        if (make_far_plan(c, P, L, found, out)) return choose_tc(c, P, L, found, out, s);
         if (c->opts.algo == FSTAT_ALGO_FARPOLY)
             return fail(c, FSTAT_EINVAL, "no far-field tile plan fits this template bank");
     }
@@ -1119,7 +1164,7 @@ int make_plan(fstat_ctx* c, Plan& out) {
     }
     if (!have) return fail(c, FSTAT_EINVAL, "no Dirichlet tile plan fits this template bank");
     out = best;
-    if (far_eligible(c) && c->have_cov) choose_tc(c, P, L, found, out);   // the rings take coverage at L = 2 only
+    if (far_eligible(c) && c->have_cov) return choose_tc(c, P, L, found, out, s);   // the rings take coverage at L = 2 only
     return FSTAT_OK;
 }
 
@@ -1179,6 +1224,9 @@ int flag_status(fstat_ctx* c) {
 
 // The bins the path reads: the whitened copy when the noise floor is on.
 const float2* work_bins(const fstat_ctx* c) { return c->nf_half > 0 ? c->d_bins_w : c->d_bins; }
+const void* form_bins(const fstat_ctx* c) {
+    return c->opts.bins_form == FSTAT_BINS_C64 ? (const void*)work_bins(c) : (const void*)c->d_bins16;
+}
 
 int refresh_sft_state(fstat_ctx* c, cudaStream_t s) {
     if (!c->sft_dirty) return FSTAT_OK;
@@ -1220,6 +1268,24 @@ int refresh_sft_state(fstat_ctx* c, cudaStream_t s) {
     c->sft_dirty = false;
     c->tab_dirty = true;
     c->gt_dirty = true;
+    c->tc_band_loud = -1;
+    return FSTAT_OK;
+}
+
+// Refresh the per-SFT state and the plan.  New bins under an unchanged bank keep
+// the plan, unless their range decides otherwise on the tensor-core form.
+int ensure_plan(fstat_ctx* c, cudaStream_t s) {
+    int rc;
+    if ((rc = refresh_sft_state(c, s)) != FSTAT_OK) return rc;
+    if (c->plan_valid && c->plan.tc_by_range && c->tc_band_loud < 0) {
+        bool fits;
+        int lo, hi;
+        if ((rc = tc_range(c, s, &fits, &lo, &hi)) != FSTAT_OK) return rc;
+        if (fits != c->plan.tc || lo != c->plan.tc_lo || hi != c->plan.tc_hi) c->plan_valid = false;
+    }
+    if (c->plan_valid) return FSTAT_OK;
+    if ((rc = make_plan(c, c->plan, s)) != FSTAT_OK) return rc;
+    c->plan_valid = true;
     return FSTAT_OK;
 }
 
@@ -1555,11 +1621,7 @@ int ensure_tables(fstat_ctx* c, cudaStream_t s);
 
 int prepare(fstat_ctx* c, cudaStream_t s) {
     int rc;
-    if ((rc = refresh_sft_state(c, s)) != FSTAT_OK) return rc;
-    if (!c->plan_valid) {
-        if ((rc = make_plan(c, c->plan)) != FSTAT_OK) return rc;
-        c->plan_valid = true;
-    }
+    if ((rc = ensure_plan(c, s)) != FSTAT_OK) return rc;
     const size_t n_meta = (size_t)c->n_sky * c->n_sft;
     const size_t n_base = n_meta * c->n_fdot;
     const size_t n_twoF = (size_t)c->n_sky * c->n_fdot * c->n_f;
@@ -1613,16 +1675,17 @@ int ensure_tables(fstat_ctx* c, cudaStream_t s) {
                            kTcCols)) !=
             FSTAT_OK)
             return rc;
-        if (c->gt_dirty || c->gt_nblk != n_blk || c->gt_xoff != xoff) {
+        if (c->gt_dirty || c->gt_nblk != n_blk || c->gt_xoff != xoff || c->gt_lo != c->plan.tc_lo || c->gt_hi != c->plan.tc_hi) {
             if ((rc = grow(c, &c->d_gtab, c->cap_gtab, (size_t)c->n_sft * n_blk * 256)) != FSTAT_OK) return rc;
             if ((rc = grow(c, &c->d_inv, c->cap_inv, (size_t)c->n_sft)) != FSTAT_OK) return rc;
-            const void* bins = c->opts.bins_form == FSTAT_BINS_C64 ? (const void*)work_bins(c) : (const void*)c->d_bins16;
-            CUDA_TRY(c, launch_tc_tables(bins, c->opts.bins_form, c->row, c->n_sft, c->n_bins, n_blk, xoff, c->d_gtab,
-                                         c->d_inv, s));
+            CUDA_TRY(c, launch_tc_tables(form_bins(c), c->opts.bins_form, c->row, c->n_sft, c->plan.tc_lo, c->plan.tc_hi, n_blk,
+                                         xoff, c->d_gtab, c->d_inv, s));
             c->launches += 1;
             c->gt_dirty = false;
             c->gt_nblk = n_blk;
             c->gt_xoff = xoff;
+            c->gt_lo = c->plan.tc_lo;
+            c->gt_hi = c->plan.tc_hi;
         }
         return FSTAT_OK;
     }
@@ -1631,7 +1694,7 @@ int ensure_tables(fstat_ctx* c, cudaStream_t s) {
         (c->tab_dirty || c->tab_npos != c->n_pos || c->tab_xoff != c->far_xoff || c->tab_sinc != c->plan.sinc ||
          (c->plan.sinc && c->tab_split != (c->plan.L == 2)))) {
         const size_t n_tab = (size_t)c->n_sft * c->n_pos;
-        const void* bins = c->opts.bins_form == FSTAT_BINS_C64 ? (const void*)work_bins(c) : (const void*)c->d_bins16;
+        const void* bins = form_bins(c);
         if (c->plan.sinc) {
             if ((rc = grow(c, &c->d_pcoef, c->cap_pcoef, 6 * n_tab)) != FSTAT_OK) return rc;
             CUDA_TRY(c, launch_sinc_tables(bins, c->opts.bins_form, c->row, c->n_sft, c->n_bins, c->sgam, c->d_pcoef,
@@ -1695,7 +1758,7 @@ TimingParams timing_params(const fstat_ctx* c, int n_sky) {
 DirichletParams dirichlet_params(const fstat_ctx* c) {
     const Plan& pl = c->plan;
     DirichletParams dp{};
-    dp.bins = c->opts.bins_form == FSTAT_BINS_C64 ? (const void*)work_bins(c) : (const void*)c->d_bins16;
+    dp.bins = form_bins(c);
     dp.row = c->row;
     dp.k_lo = c->k_lo;
     dp.n_bins = c->n_bins;
@@ -1955,11 +2018,9 @@ int fstat_get_error_flags(fstat_ctx* c, int32_t* flags) {
 int fstat_get_plan(fstat_ctx* c, int32_t* out) {
     if (!c || !out) return FSTAT_EINVAL;
     if (!c->have_sfts || !c->have_templates) return fail(c, FSTAT_ESTATE, "load SFTs and set templates first");
-    if (!c->plan_valid) {
-        int rc = make_plan(c, c->plan);
-        if (rc != FSTAT_OK) return rc;
-        c->plan_valid = true;
-    }
+    if (set_device(c) != FSTAT_OK) return FSTAT_ECUDA;
+    const int rc = ensure_plan(c, c->stream);
+    if (rc != FSTAT_OK) return rc;
     const Plan& p = c->plan;
     const int v[8] = {p.P, p.L, p.M, p.W, p.C, p.lg_row, p.w_pairs, p.far ? kFarIdBase + p.variant : p.variant};
     std::memcpy(out, v, sizeof(v));
@@ -2125,7 +2186,7 @@ int fstat_autotune(fstat_ctx* c, void* cuda_stream, int32_t* out) {
             c->opts.tile_m = M;
             c->opts.sft_chunk = C;
             c->plan_valid = false;
-            if (make_plan(c, c->plan) != FSTAT_OK) continue;
+            if (make_plan(c, c->plan, s) != FSTAT_OK) continue;
             c->plan_valid = true;
             if (c->plan.C != C) continue;   // round size capped by shared memory
             if (c->plan.sky_perm) continue;   // the slice takes the first sky points, not an order's groups
@@ -2205,9 +2266,10 @@ int fstat_batch_add(fstat_ctx* c, const fstat_workunit* wu, int32_t* wu_id) {
     // the persistent kernels exist for the direct and the ring forms: a workunit
     // the far-field form would stage in rounds runs the direct form, alone or batched
     Plan pl;
-    if (make_plan(w, pl) == FSTAT_OK && (pl.rows || pl.two)) {   // no persistent form of these: the one-row ring
+    rc = refresh_sft_state(w, w->stream);
+    if (rc == FSTAT_OK && make_plan(w, pl, w->stream) == FSTAT_OK && (pl.rows || pl.two)) {   // no persistent form of these: the one-row ring
         w->opts.algo = FSTAT_ALGO_SINCPOLY;
-        if (make_plan(w, pl) != FSTAT_OK) pl = Plan{};
+        if (make_plan(w, pl, w->stream) != FSTAT_OK) pl = Plan{};
     }
     if (pl.far && !pl.tc && (!pl.ring || pl.L != 2)) w->opts.algo = FSTAT_ALGO_DIRECT;
     w->plan_valid = false;

@@ -303,8 +303,12 @@ cudaError_t launch_far_tables(const void* bins, int form, long long row, int n_s
 cudaError_t launch_sinc_tables(const void* bins, int form, long long row, int n_sft, int n_bins,
                                const SincGamma& gam, float4* pcoef, int n_pos, int xoff, bool split,
                                cudaStream_t s);
-cudaError_t launch_tc_tables(const void* bins, int form, long long row, int n_sft, int n_bins, int n_blk, int xoff,
+// Tables of the bins lo .. hi - 1 (zeros elsewhere).
+cudaError_t launch_tc_tables(const void* bins, int form, long long row, int n_sft, int lo, int hi, int n_blk, int xoff,
                              unsigned char* gtab, float* inv_scale, cudaStream_t s);
+// *flag |= 1 where the windows inside lo .. hi - 1 span a range the tables do not hold.
+cudaError_t launch_tc_range(const void* bins, int form, long long row, int n_sft, int n_bins, int lo, int hi, int* flag,
+                            cudaStream_t s);
 int tc_blocks(int n_tiles, int n_colb, int n_sft, int sms);   // blocks of the kernel
 int tc_launches(const TcParams& p);                            // kernels that launch_dirichlet_tc launches
 cudaError_t launch_dirichlet_tc(const TcParams& p, cudaStream_t s);

@@ -736,61 +736,58 @@ __global__ void __launch_bounds__(kThreads, 1) dirichlet_tc_kernel(const TcParam
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t td = tbase + (n & 1) * (2 * kCols);
+                bool any = true;   // some column of the warp is covered
                 if (COV && (cvr[n & 7].x > 32 * h * p.n_sub || cvr[n & 7].y < (32 * h + 32) * p.n_sub)) {
                     // not all of the warp's columns are covered: zeros into the others' window sums
                     const int2 cv = cvr[n & 7];
-                    if (cv.x >= (32 * h + 32) * p.n_sub || cv.y <= 32 * h * p.n_sub) {   // none: the sums stay
-                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                        __syncwarp();
-                        if (lane == 0) {
-                            mbar_arrive(d_free(n));
-                            mbar_arrive(r_free(n));
-                        }
-                        continue;
-                    }
-                    const int item = (int)((run_first(p) + n) / p.n_sft);
-                    const int jr = 32 * h * p.n_sub + ((item % p.n_tiles) * p.rt + row) % p.rps % p.n_sub;
+                    any = cv.x < (32 * h + 32) * p.n_sub && cv.y > 32 * h * p.n_sub;   // none: the sums stay
+                    if (any) {
+                        const int item = (int)((run_first(p) + n) / p.n_sft);
+                        const int jr = 32 * h * p.n_sub + ((item % p.n_tiles) * p.rt + row) % p.rps % p.n_sub;
 #pragma unroll 1
-                    for (int ch = 0; ch < 4; ++ch) {
-                        float u[16];
-                        tmem_ld16(td + 16 * ch, u);
-                        tmem_wait16(u);
+                        for (int ch = 0; ch < 4; ++ch) {
+                            float u[16];
+                            tmem_ld16(td + 16 * ch, u);
+                            tmem_wait16(u);
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) {
-                            const int j = jr + p.n_sub * (8 * ch + 4 * (e >> 3) + (e & 3));
-                            u[e] = j >= cv.x && j < cv.y ? u[e] : 0.0f;
+                            for (int e = 0; e < 16; ++e) {
+                                const int j = jr + p.n_sub * (8 * ch + 4 * (e >> 3) + (e & 3));
+                                u[e] = j >= cv.x && j < cv.y ? u[e] : 0.0f;
+                            }
+                            tmem_st16(td + 16 * ch, u);
                         }
-                        tmem_st16(td + 16 * ch, u);
+                        tmem_wait_st();
                     }
-                    tmem_wait_st();
                 }
-                float v[2][16];
-                tmem_ld16(td, v[0]);
-                tmem_wait16(v[0]);
+                if (!COV || any) {
+                    float v[2][16];
+                    tmem_ld16(td, v[0]);
+                    tmem_wait16(v[0]);
 #pragma unroll
-                for (int ch = 0; ch < 4; ++ch) {   // eight columns: twice four real parts, four imaginary parts
-                    float (&cv)[16] = v[ch & 1];
-                    if (ch < 3) tmem_ld16(td + 16 * (ch + 1), v[(ch + 1) & 1]);
+                    for (int ch = 0; ch < 4; ++ch) {   // eight columns: twice four real parts, four imaginary parts
+                        float (&cv)[16] = v[ch & 1];
+                        if (ch < 3) tmem_ld16(td + 16 * (ch + 1), v[(ch + 1) & 1]);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int o = 8 * (q >> 1) + 2 * (q & 1), i = 4 * ch + q;
-                        const float2 pr = make_float2(cv[o], cv[o + 1]), pi = make_float2(cv[o + 4], cv[o + 5]);
-                        float2& wr = tr[q & 1];
-                        float2& wi = ti[q & 1];
-                        const float2 nwi = make_float2(-wi.x, -wi.y);
-                        const float2 zr = __ffma2_rn(wr, pr, __fmul2_rn(nwi, pi));
-                        const float2 zi = __ffma2_rn(wr, pi, __fmul2_rn(wi, pr));
-                        far[i] = __ffma2_rn(a2, zr, far[i]);
-                        fai[i] = __ffma2_rn(a2, zi, fai[i]);
-                        fbr[i] = __ffma2_rn(b2, zr, fbr[i]);
-                        fbi[i] = __ffma2_rn(b2, zi, fbi[i]);
-                        if (i < 14) {   // four columns on
-                            const float2 nr = __ffma2_rn(wr, rr, __fmul2_rn(wi, nri));
-                            wi = __ffma2_rn(wr, ri, __fmul2_rn(wi, rr));
-                            wr = nr;
+                        for (int q = 0; q < 4; ++q) {
+                            const int o = 8 * (q >> 1) + 2 * (q & 1), i = 4 * ch + q;
+                            const float2 pr = make_float2(cv[o], cv[o + 1]), pi = make_float2(cv[o + 4], cv[o + 5]);
+                            float2& wr = tr[q & 1];
+                            float2& wi = ti[q & 1];
+                            const float2 nwi = make_float2(-wi.x, -wi.y);
+                            const float2 zr = __ffma2_rn(wr, pr, __fmul2_rn(nwi, pi));
+                            const float2 zi = __ffma2_rn(wr, pi, __fmul2_rn(wi, pr));
+                            far[i] = __ffma2_rn(a2, zr, far[i]);
+                            fai[i] = __ffma2_rn(a2, zi, fai[i]);
+                            fbr[i] = __ffma2_rn(b2, zr, fbr[i]);
+                            fbi[i] = __ffma2_rn(b2, zi, fbi[i]);
+                            if (i < 14) {   // four columns on
+                                const float2 nr = __ffma2_rn(wr, rr, __fmul2_rn(wi, nri));
+                                wi = __ffma2_rn(wr, ri, __fmul2_rn(wi, rr));
+                                wr = nr;
+                            }
                         }
+                        if (ch < 3) tmem_wait16(v[(ch + 1) & 1]);
                     }
-                    if (ch < 3) tmem_wait16(v[(ch + 1) & 1]);
                 }
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();

@@ -344,8 +344,11 @@ int fstat_take_kernel_time(fstat_ctx *ctx, double *ms_dirichlet, double *ms_tota
  * points, a few waves of blocks) and keep the fastest as the context's tile
  * choice for later computes.  out[4] (host, may be NULL) receives
  * (M, sft_chunk, warps, best kernel time on the slice in microseconds).
- * A batch context (workunits only) tunes on its largest workunit and gives
- * every workunit that M; each keeps the stage count its own plan chooses.
+ * The tensor-core form (see AUTO) has no tiles to tune: out then holds its time
+ * on the slice beside the plan it replaces, and nothing changes.
+ * A batch context (workunits only) tunes on its largest workunit that is not
+ * on the tensor-core form and gives every such workunit that M; each keeps the
+ * stage count its own plan chooses.
  * Synchronises.  Errors: ESTATE (no SFTs or templates). */
 int fstat_autotune(fstat_ctx *ctx, void *cuda_stream, int32_t *out);
 

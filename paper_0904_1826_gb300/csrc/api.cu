@@ -2098,24 +2098,35 @@ int fstat_take_kernel_time(fstat_ctx* c, double* ms_dirichlet, double* ms_total,
 int fstat_autotune(fstat_ctx* c, void* cuda_stream, int32_t* out) {
     if (!c) return FSTAT_EINVAL;
     c->err.clear();
-    // a context holding only workunits tunes on its largest one and applies its
-    // templates per thread to all; each workunit keeps the planner's stage count,
-    // which follows its own table width and residency (one stage count for all
-    // cost up to 60 % on workunits whose stages then left one block per SM)
+    // a context holding only workunits tunes on the largest one that has tiles to
+    // tune (not the tensor-core form, whose plan's M is that of a kernel that does
+    // not run) and applies its templates per thread to all that have; each workunit
+    // keeps the planner's stage count, which follows its own table width and
+    // residency (one stage count for all cost up to 60 % on workunits whose stages
+    // then left one block per SM)
     if ((!c->have_sfts || !c->have_templates) && !c->wus.empty()) {
-        fstat_ctx* big = c->wus[0];
-        for (fstat_ctx* w : c->wus)
-            if ((double)w->n_sky * w->n_f * w->n_fdot * w->n_sft > (double)big->n_sky * big->n_f * big->n_fdot * big->n_sft)
-                big = w;
-        int32_t o[4];
-        int rc = fstat_autotune(big, cuda_stream, o);
-        if (rc != FSTAT_OK) return fail(c, rc, "autotune: %s", big->err.c_str());
-        for (fstat_ctx* w : c->wus) {   // the tuned workunit too returns to the caller's stage count
-            w->opts.tile_m = o[0];
-            w->opts.sft_chunk = c->opts.sft_chunk;
-            w->plan_valid = false;
+        if (set_device(c) != FSTAT_OK) return FSTAT_ECUDA;
+        int rc;
+        fstat_ctx *big = nullptr, *tuned = nullptr;
+        auto size = [](const fstat_ctx* w) { return (double)w->n_sky * w->n_f * w->n_fdot * w->n_sft; };
+        for (fstat_ctx* w : c->wus) {
+            if ((rc = ensure_plan(w, (cudaStream_t)cuda_stream)) != FSTAT_OK) return fail(c, rc, "autotune: %s", w->err.c_str());
+            if (!big || size(w) > size(big)) big = w;
+            if (!w->plan.tc && (!tuned || size(w) > size(tuned))) tuned = w;
         }
-        c->opts.tile_m = o[0];
+        if (tuned) big = tuned;
+        int32_t o[4];
+        rc = fstat_autotune(big, cuda_stream, o);
+        if (rc != FSTAT_OK) return fail(c, rc, "autotune: %s", big->err.c_str());
+        if (tuned) {
+            for (fstat_ctx* w : c->wus) {   // the tuned workunit too returns to the caller's stage count
+                if (w != tuned && w->plan.tc) continue;
+                w->opts.tile_m = o[0];
+                w->opts.sft_chunk = c->opts.sft_chunk;
+                w->plan_valid = false;
+            }
+            c->opts.tile_m = o[0];
+        }
         c->graph_valid = false;
         if (out) std::memcpy(out, o, sizeof(o));
         return FSTAT_OK;

@@ -229,6 +229,8 @@ struct fstat_ctx {
     int n_groups = 0;
     cudaEvent_t bev0 = nullptr, bev1 = nullptr;
     long long launches_per_graph = 0;
+    float4* d_batch_tcs = nullptr;    // scratch of the batch's tensor-core workunits
+    size_t cap_batch_tcs = 0;
     std::vector<int> batch_order;     // grouped position -> workunit index
     int* d_fstart = nullptr;          // patch frequency starts
     size_t cap_fstart = 0;
@@ -1285,6 +1287,19 @@ int ensure_plan(fstat_ctx* c, cudaStream_t s) {
     }
     if (c->plan_valid) return FSTAT_OK;
     if ((rc = make_plan(c, c->plan, s)) != FSTAT_OK) return rc;
+    if (c->batch_member) {
+        // the persistent kernels exist for the direct and the one-row L = 2 ring forms:
+        // a workunit of another one runs the ring or the direct form, alone or batched
+        const Plan& pl = c->plan;
+        if (pl.rows || pl.two) {
+            c->opts.algo = FSTAT_ALGO_SINCPOLY;
+            if ((rc = make_plan(c, c->plan, s)) != FSTAT_OK) return rc;
+        }
+        if (pl.far && !pl.tc && (!pl.ring || pl.L != 2 || pl.rows || pl.two)) {
+            c->opts.algo = FSTAT_ALGO_DIRECT;
+            if ((rc = make_plan(c, c->plan, s)) != FSTAT_OK) return rc;
+        }
+    }
     c->plan_valid = true;
     return FSTAT_OK;
 }
@@ -1670,11 +1685,6 @@ int ensure_tables(fstat_ctx* c, cudaStream_t s) {
         far_extent(c, kTcCols + 4 * kTcBlkMax + 8, &xoff, &n_pos);
         xoff = (xoff + 4 + 3) & ~3;
         const int n_blk = (n_pos + 8 + 3) / 4;
-        if ((rc = grow(c, &c->d_tcs, c->cap_tcs,
-                       (size_t)tc_blocks(c->plan.tc_tiles, c->plan.tc_colb, c->n_sft, current_sm_count()) * kTcSlots * kTcRows *
-                           kTcCols)) !=
-            FSTAT_OK)
-            return rc;
         if (c->gt_dirty || c->gt_nblk != n_blk || c->gt_xoff != xoff || c->gt_lo != c->plan.tc_lo || c->gt_hi != c->plan.tc_hi) {
             if ((rc = grow(c, &c->d_gtab, c->cap_gtab, (size_t)c->n_sft * n_blk * 256)) != FSTAT_OK) return rc;
             if ((rc = grow(c, &c->d_inv, c->cap_inv, (size_t)c->n_sft)) != FSTAT_OK) return rc;
@@ -1713,6 +1723,18 @@ int ensure_tables(fstat_ctx* c, cudaStream_t s) {
         c->tab_split = c->plan.L == 2;
     }
     return FSTAT_OK;
+}
+
+// Scratch of the tensor-core kernel (float4).  A context's own computes use its own;
+// the workunits of a batch, launched one after another, share their parent's.
+size_t tc_scratch(const fstat_ctx* c) {
+    return c->plan.tc ? (size_t)tc_blocks(c->plan.tc_tiles, c->plan.tc_colb, c->n_sft, current_sm_count()) * kTcSlots * kTcRows *
+                            kTcCols
+                      : 0;
+}
+
+int ensure_scratch(fstat_ctx* c) {
+    return c->plan.tc ? grow(c, &c->d_tcs, c->cap_tcs, tc_scratch(c)) : FSTAT_OK;
 }
 
 TimingParams timing_params(const fstat_ctx* c, int n_sky) {
@@ -1795,7 +1817,7 @@ DirichletParams dirichlet_params(const fstat_ctx* c) {
     return dp;
 }
 
-TcParams tc_params(const fstat_ctx* c) {
+TcParams tc_params(const fstat_ctx* c, float4* scratch) {
     const Plan& pl = c->plan;
     TcParams t{};
     t.gtab = c->d_gtab;
@@ -1810,7 +1832,7 @@ TcParams tc_params(const fstat_ctx* c) {
     t.cov = c->have_cov ? c->d_cov : nullptr;
     t.comb_j = c->d_comb_j;
     t.twoF = c->d_twoF;
-    t.scratch = c->d_tcs;
+    t.scratch = scratch;
     t.err = c->d_err;
     t.n_sft = c->n_sft;
     t.n_sky = c->n_sky;
@@ -1837,13 +1859,15 @@ bool tables_match(const fstat_ctx* c, const Plan& pl) {
            c->n_pos == n_pos && c->far_xoff == xoff;
 }
 
+cudaError_t launch_tc(const fstat_ctx* c, float4* scratch, cudaStream_t s) {
+    if (!scratch || c->gt_dirty || (c->plan.tc_perm && c->perm_on_device != 2)) return cudaErrorInvalidValue;
+    return launch_dirichlet_tc(tc_params(c, scratch), s);
+}
+
 cudaError_t launch_dir(const fstat_ctx* c, const DirichletParams& dp, long long grid, cudaStream_t s) {
     const Plan& pl = c->plan;
     const int threads = pl.W * 32;
-    if (pl.tc) {
-        if (c->gt_dirty || (pl.tc_perm && c->perm_on_device != 2)) return cudaErrorInvalidValue;
-        return launch_dirichlet_tc(tc_params(c), s);
-    }
+    if (pl.tc) return launch_tc(c, c->d_tcs, s);
     if (pl.far) {
         if (!tables_match(c, pl)) return cudaErrorInvalidValue;
         return launch_dirichlet_far(pl.variant, dp, threads, pl.smem, grid, s);
@@ -1876,6 +1900,7 @@ int fstat_compute(fstat_ctx* c, void* cuda_stream) {
     c->stream = s;
     int rc;
     if ((rc = prepare(c, s)) != FSTAT_OK) return rc;
+    if ((rc = ensure_scratch(c)) != FSTAT_OK) return rc;
     CUDA_TRY(c, cudaMemsetAsync(c->d_err, 0, sizeof(int) * 3, s));
     const int slot = c->n_timed % kTimedRing;
     CUDA_TRY(c, cudaEventRecord(c->ev_a[slot], s));
@@ -1888,7 +1913,7 @@ int fstat_compute(fstat_ctx* c, void* cuda_stream) {
     cudaError_t e = launch_dir(c, dirichlet_params(c), c->plan.grid, s);
     if (e != cudaSuccess) return fail(c, FSTAT_ECUDA, "Dirichlet launch: %s", cudaGetErrorString(e));
     CUDA_TRY(c, cudaEventRecord(c->ev_c[slot], s));
-    c->launches += 1 + (c->plan.tc ? tc_launches(tc_params(c)) : 1);   // timing + Dirichlet
+    c->launches += 1 + (c->plan.tc ? tc_launches(tc_params(c, nullptr)) : 1);   // timing + Dirichlet
     if ((rc = enqueue_topk(c, s)) != FSTAT_OK) return rc;
     CUDA_TRY(c, cudaEventRecord(c->ev_d[slot], s));
     c->n_timed++;
@@ -2141,12 +2166,13 @@ int fstat_autotune(fstat_ctx* c, void* cuda_stream, int32_t* out) {
     c->opts.sft_chunk = 0;
     c->plan_valid = false;
     int rc = prepare(c, s);
+    if (rc == FSTAT_OK) rc = ensure_scratch(c);
     if (rc != FSTAT_OK) {
         c->opts = saved;
         return rc;
     }
     if (c->plan.tc) {   // nothing to tune: one tile shape; its time on a slice of about four waves
-        TcParams t = tc_params(c);
+        TcParams t = tc_params(c, c->d_tcs);
         t.n_tiles = std::min(t.n_tiles, std::max(1, 4 * current_sm_count() / t.n_colb));
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
@@ -2274,17 +2300,6 @@ int fstat_batch_add(fstat_ctx* c, const fstat_workunit* wu, int32_t* wu_id) {
         fstat_destroy(w);
         return rc;
     }
-    // the persistent kernels exist for the direct and the ring forms: a workunit
-    // the far-field form would stage in rounds runs the direct form, alone or batched
-    Plan pl;
-    rc = refresh_sft_state(w, w->stream);
-    if (rc == FSTAT_OK && make_plan(w, pl, w->stream) == FSTAT_OK && (pl.rows || pl.two)) {   // no persistent form of these: the one-row ring
-        w->opts.algo = FSTAT_ALGO_SINCPOLY;
-        if (make_plan(w, pl, w->stream) != FSTAT_OK) pl = Plan{};
-    }
-    if (pl.far && !pl.tc && (!pl.ring || pl.L != 2)) w->opts.algo = FSTAT_ALGO_DIRECT;
-    w->plan_valid = false;
-    w->err.clear();
     c->wus.push_back(w);
     c->graph_valid = false;
     c->batch_ran = false;
@@ -2312,7 +2327,7 @@ int fstat_batch_clear(fstat_ctx* c) {
     if (c->graph) cudaGraphDestroy(c->graph);
     c->graph_exec = nullptr;
     c->graph = nullptr;
-    void* ptrs[] = {c->d_banks, c->d_prefix, c->d_rem_init, c->d_rem, c->d_queue, c->d_done};
+    void* ptrs[] = {c->d_banks, c->d_prefix, c->d_rem_init, c->d_rem, c->d_queue, c->d_done, c->d_batch_tcs};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     c->d_banks = nullptr;
@@ -2321,6 +2336,8 @@ int fstat_batch_clear(fstat_ctx* c) {
     c->d_rem = nullptr;
     c->d_queue = nullptr;
     c->d_done = nullptr;
+    c->d_batch_tcs = nullptr;
+    c->cap_batch_tcs = 0;
     c->graph_valid = false;
     c->batch_ran = false;
     return FSTAT_OK;
@@ -2417,11 +2434,11 @@ int enqueue_batch(fstat_ctx* c, const std::vector<int>& order, const std::vector
     for (int k = 0; k < n; ++k) {   // tensor-core workunits: each fills the SMs by itself
         fstat_ctx* w = c->wus[order[k]];
         if (!w->plan.tc) continue;
-        cudaError_t e = launch_dir(w, DirichletParams{}, 0, s);
+        cudaError_t e = launch_tc(w, c->d_batch_tcs, s);
         if (e != cudaSuccess) return fail(c, FSTAT_ECUDA, "batch Dirichlet launch: %s", cudaGetErrorString(e));
         stamp_kernel<<<1, 1, 0, s>>>(c->d_done + k);
         CUDA_TRY(c, cudaGetLastError());
-        c->launches += 1 + tc_launches(tc_params(w));
+        c->launches += 1 + tc_launches(tc_params(w, nullptr));
     }
     for (size_t g = 1; g < groups.size(); ++g) CUDA_TRY(c, cudaStreamWaitEvent(s, c->side_events[g], 0));
     for (fstat_ctx* w : c->wus) {
@@ -2443,16 +2460,17 @@ int fstat_batch_compute(fstat_ctx* c, void* cuda_stream) {
     cudaStream_t s = (cudaStream_t)cuda_stream;
     c->stream = s;
     const int n = (int)c->wus.size();
+    size_t scratch = 0;
     for (fstat_ctx* w : c->wus) {
         w->stream = s;
         int rc = prepare(w, s);
         if (rc != FSTAT_OK) return fail(c, rc, "workunit: %s", w->err.c_str());
-        if (w->plan.far && !w->plan.tc && (!w->plan.ring || w->plan.L != 2 || w->plan.rows || w->plan.two)) {   // persistent: direct, one-row L = 2 ring
-            w->opts.algo = FSTAT_ALGO_DIRECT;
-            w->plan_valid = false;
-            c->graph_valid = false;
-            if ((rc = prepare(w, s)) != FSTAT_OK) return fail(c, rc, "workunit: %s", w->err.c_str());
-        }
+        scratch = std::max(scratch, tc_scratch(w));
+    }
+    if (scratch > c->cap_batch_tcs) {
+        c->graph_valid = false;
+        const int rc = grow(c, &c->d_batch_tcs, c->cap_batch_tcs, scratch);
+        if (rc != FSTAT_OK) return rc;
     }
     if (!c->bev0) {
         cudaEventCreate(&c->bev0);

@@ -61,3 +61,52 @@ def test_batch_autotune_of_tensor_workunits_only_changes_nothing(lib):
             np.testing.assert_array_equal(lib.fstat_batch_get_2f(g.ctx, i, 0, w.n_templates), alone[i][0])
     finally:
         g.close()
+
+
+def test_loud_fine_grid_workunit_alone_and_batched(lib):
+    """A fine-grid workunit whose bins keep it off the tensor cores falls back to a form
+    with a persistent kernel, the same alone and in the batch; a quiet one does not."""
+    w = _dense(903, n_sft=8, n_f=511, n_fdot=1, n_bins=120, df_bins=0.125)
+    quiet = [d.bins for d in w.detectors]
+    loud = [b.copy() for b in quiet]
+    loud[0][:, 60] += np.complex64(1e9)
+    g = lib.FStat(0, topk=20)
+    try:
+        for bins in (loud, quiet):
+            lib.fstat_batch_add(g.ctx, w, bins)
+        one = []
+        for i in (0, 1):
+            lib.fstat_batch_compute_one(g.ctx, i)
+            one.append(lib.fstat_batch_get_2f(g.ctx, i, 0, w.n_templates))
+        for _ in range(2):
+            lib.fstat_batch_compute(g.ctx)
+            for i in (0, 1):
+                np.testing.assert_array_equal(lib.fstat_batch_get_2f(g.ctx, i, 0, w.n_templates), one[i])
+    finally:
+        g.close()
+    np.testing.assert_array_equal(one[1], _alone(lib, w)[0])
+
+
+def test_tensor_workunits_share_one_scratch(lib):
+    """Device memory of a batch: a tensor workunit more costs its own tables and 2F, not
+    another scratch area (59.8 MB on 152 SMs; the tables and 2F here take 15 MB)."""
+    import torch
+    w = _dense(600, **TENSOR)
+    ref, rows = _alone(lib, w)
+    assert rows > 0
+    used = []
+    for n in (2, 6):
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        g = lib.FStat(0, topk=20)
+        try:
+            for _ in range(n):
+                lib.fstat_batch_add(g.ctx, w)
+            for _ in range(2):
+                lib.fstat_batch_compute(g.ctx)
+            for i in range(n):
+                np.testing.assert_array_equal(lib.fstat_batch_get_2f(g.ctx, i, 0, w.n_templates), ref)
+            used.append(free - torch.cuda.mem_get_info()[0])
+        finally:
+            g.close()
+    assert used[1] - used[0] < 4 * 40e6, used

@@ -12,11 +12,13 @@ basis kernel, the Dirichlet kernel with fused 2F, and the toplist selection.
   python bench.py --coverage F | --noise-floor W | --algo ...   (variants)
 
 The JSON line's `roofline` is the Dirichlet kernel's ALU bound (100 flop per
-pair of the direct sum, peak from the queried SM count), with the DRAM traffic
-and, for the table forms, the shared-memory bound (`roofline.shared_memory`)
-taken from the committed ncu summary while it matches the kernel source.
-`plain_fp32` times the plain FP32 form (direct Dirichlet sum) on the same
-workunit; `twoF_error` gives max and p99 |GPU 2F - oracle 2F| of both forms
+pair of the direct sum, 24 in the tensor-core form; peak from the queried SM
+count), with the DRAM traffic and, for the table forms, the shared-memory bound
+(`roofline.shared_memory`), for the tensor-core form the issue slots
+(`roofline.issue`), taken from the committed ncu summary while it matches the
+kernel source.  `plain_fp32` times the plain FP32 form (direct Dirichlet sum) on
+the same workunit; `twoF_error` gives max and p99 |GPU 2F - oracle 2F| of both
+forms (the chosen one on the whole bank, as timed)
 on the CPU baseline's sample (16 sky points x 1800 f x 10 fdot x 2400 SFTs,
 signals added by the FP64 oracle), which the plain-C FP64 oracle times on
 every host core (`cpu_baseline`, also one core); `--impl reference` times the
@@ -45,6 +47,9 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 FLOP_PER_PAIR = 100.0          # direct-sum FP32 work of one template.SFT pair: 16 bins x (4 + 1) + 20 per-pair constants
+# FP32 work of a pair in the tensor-core form, whose 16 taps are not FP32 work: twiddle,
+# product, Fa and Fb 19, and a row's weights (330 a row and SFT) over its 64 columns 5
+FLOP_PER_PAIR_TENSOR = 24.0
 FP32_LANES = 128
 METRIC = "template·SFT pairs/s (2F) on 1 GB300, chosen vs plain FP32 form at stated 2F error"
 KERNEL_SOURCES = {"direct": ["fstat_internal.cuh", "dirichlet.cuh", "dirichlet_c64.cu", "dirichlet_f16.cu",
@@ -57,6 +62,20 @@ KERNEL_SOURCES = {"direct": ["fstat_internal.cuh", "dirichlet.cuh", "dirichlet_c
 KERNEL_NAMES = {"direct": "dirichlet_kernel", "farpoly": "dirichlet_far_kernel",
                 "sincpoly": "dirichlet_far_ring_kernel", "sincrows": "dirichlet_rows_kernel",
                 "sincpairs": "dirichlet_ring2_kernel", "tensor": "dirichlet_tc_kernel"}
+
+
+def kernel_of(plan: dict, tensor_rows: int):
+    """(form, kernel) that runs under this plan; with the tensor-core form the plan is
+    that of the kernel it replaces."""
+    if tensor_rows > 0:
+        return "tensor", KERNEL_NAMES["tensor"]
+    vid = plan.get("variant", 0)
+    form = algo_of(vid)
+    return form, KERNEL_NAMES[form] if vid < 107 or vid >= 120 else "dirichlet_far_ring_kernel"
+
+
+def flop_per_pair(tensor_rows: int) -> float:
+    return FLOP_PER_PAIR_TENSOR if tensor_rows > 0 else FLOP_PER_PAIR
 
 
 def parse():
@@ -306,6 +325,32 @@ def twoF_error_stats(got, ref) -> dict:
             "max_2F": float(ref.max())}
 
 
+def gpu_2f_error(w, pick, bins, sub, ref, device, stream, **chosen) -> dict:
+    """The GPU's 2F at the CPU baseline's sample (the sky points `pick`, signals added by
+    the oracle) against the oracle's all-core run.  The chosen form computes the whole
+    bank, as timed: a form can depend on the bank, and the tensor-core form does.  The
+    plain FP32 form, which does not, computes the sample's own bank."""
+    import dataclasses
+    import paper_0904_1826_gb300 as fs
+    per_sky = w.bank.n_fdot * w.bank.n_f
+    out = {}
+    for name, wl, opts in (("chosen", w, chosen),
+                           ("plain_fp32", dataclasses.replace(w, bank=sub), dict(bins_form="c64", algo="direct"))):
+        g = fs.FStat(device, dterms=w.dterms, topk=10, **opts)
+        try:
+            g.load_workload(wl, bins_override=bins)
+            g.compute(stream)
+            got = (np.concatenate([g.twoF(i * per_sky, per_sky) for i in pick]) if wl is w else g.twoF())
+            st = twoF_error_stats(got, ref)
+            plan = g.plan()
+            st["variant"] = plan["variant"]
+            st["kernel"] = kernel_of(plan, g.tensor_tiles()["rows"])[1]
+            out[name] = st
+        finally:
+            g.close()
+    return out
+
+
 def shared_config(args) -> dict:
     """The workload description both arms print."""
     return {"workload": "plain workunit: 2 det x 1200 gapped SFT (T=1800 s), 1 Hz band at 100 Hz, "
@@ -365,7 +410,7 @@ def run_semicoherent(args):
     edges = t0 + (t1 - t0) * np.arange(args.n_seg + 1) / args.n_seg
     edges[-1] += 1.0
     bank, pad = w.bank, 8
-    segs, seg_pairs, seg_bytes = [], 0, 0
+    segs, seg_pairs, seg_flop, seg_bytes = [], 0, 0.0, 0
     for s in range(args.n_seg):
         dets = []
         for i, d in enumerate(w.detectors):
@@ -376,7 +421,9 @@ def run_semicoherent(args):
         g = fs.FStat(local_rank, topk=10, algo=args.algo)
         g.load_workload(Workload(w.name, w.T, w.k_lo, w.n_bins, w.dterms, 10, dets, bs))
         segs.append(g)
-        seg_pairs += bs.n_sky * bs.n_fdot * bs.n_f * sum(d.n_sft for d in dets)
+        n_p = bs.n_sky * bs.n_fdot * bs.n_f * sum(d.n_sft for d in dets)
+        seg_pairs += n_p
+        seg_flop += n_p * flop_per_pair(g.tensor_tiles()["rows"])
         seg_bytes += 4 * bs.n_sky * bs.n_fdot * bs.n_f
     n_t = bank.n_sky * bank.n_fdot * bank.n_f
     out = torch.empty(n_t, dtype=torch.float32, device="cuda")
@@ -430,7 +477,7 @@ def run_semicoherent(args):
             peak_gbs = float(json.load(fh)["hbm_gbs"])
     except (OSError, ValueError, KeyError):
         pass
-    achieved = FLOP_PER_PAIR * seg_pairs / (k_dir / 1e3) / 1e12
+    achieved = seg_flop / (k_dir / 1e3) / 1e12
     n_sm = int(torch.cuda.get_device_properties(local_rank).multi_processor_count)
     peak = n_sm * FP32_LANES * 2 * 2070.0 * 1e6 / 1e12
     line = {"metric": METRIC, "value": seg_pairs * args.steps / (ms / 1e3), "unit": "pairs/s", "n_gpus": 1,
@@ -758,7 +805,7 @@ def main():
             ms2, kd2, _, _ = timed_run(g2, args.steps, 1)
             name = f + ("+kahan" if kahan else "") + ("" if kahan or algo == "auto" else "/" + algo)
             forms[name] = {"value": n_pairs * args.steps / (ms2 / 1e3), "dirichlet_ms": kd2,
-                           "algo": algo_of(g2.plan()["variant"])}
+                           "algo": kernel_of(g2.plan(), g2.tensor_tiles()["rows"])[0]}
             g2.close()
 
     # the plain FP32 form (direct Dirichlet sum, FP32 bins) on the same workunit
@@ -779,17 +826,15 @@ def main():
     n_sm = int(props.multi_processor_count)
     clock_mhz = float(clocks["sm_max_mhz"]) if clocks and clocks.get("sm_max_mhz") else 2070.0
     peak = n_sm * FP32_LANES * 2 * clock_mhz * 1e6 / 1e12       # TFLOP/s, recipe unit counts, max clock
-    achieved = FLOP_PER_PAIR * n_pairs / (k_dir / 1e3) / 1e12
-    vid = plan.get("variant", 0)
-    algo_used = "tensor" if tensor_rows > 0 else algo_of(vid)   # the plan stays the ring it replaces
-    kernel_name = (KERNEL_NAMES[algo_used] if (vid < 107 or vid >= 120 or tensor_rows > 0)
-                   else "dirichlet_far_ring_kernel")
+    achieved = flop_per_pair(tensor_rows) * n_pairs / (k_dir / 1e3) / 1e12
+    algo_used, kernel_name = kernel_of(plan, tensor_rows)
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": ncu_traffic(args.form, algo_used), "kernel": kernel_name,
                 "dirichlet_ms": k_dir, "step_ms_device": k_step,
                 "peak_note": f"{n_sm} SM (queried) x {FP32_LANES} FP32 lanes x 2 flop x {clock_mhz:.0f} MHz "
                              "(maximum SM clock)"
-                             + ("; the tensor form runs the window sums on the tensor cores" if tensor_rows > 0 else "")}
+                             + (f"; {FLOP_PER_PAIR_TENSOR:.0f} FP32 flop a pair, the window sums run on the tensor cores"
+                                if tensor_rows > 0 else "")}
     if clocks and clocks.get("sm_mhz"):
         roofline["frac_at_sampled_clock"] = achieved / (n_sm * FP32_LANES * 2 * clocks["sm_mhz"] * 1e6 / 1e12)
     # the table forms are bound by shared-memory loads: that bound too, from the
@@ -801,6 +846,12 @@ def main():
         roofline["shared_memory"] = {"achieved": smem_b / (k_dir / 1e3) / 1e12, "peak": smem_peak, "unit": "TB/s",
                                      "frac": smem_b / (k_dir / 1e3) / 1e12 / smem_peak,
                                      "bytes_per_pair": ent["smem_wavefronts_per_pair"] * 128.0}
+    # the tensor-core form is nearest to its issue slots (4 a clock and SM)
+    if ent and ent.get("warp_instructions_per_pair"):
+        issued = ent["warp_instructions_per_pair"] * n_pairs / (k_dir / 1e3)
+        slots = n_sm * 4.0 * clock_mhz * 1e6
+        roofline["issue"] = {"achieved": issued / 1e9, "peak": slots / 1e9, "unit": "G warp instructions/s",
+                             "frac": issued / slots}
     config = shared_config(args)
     config["pairs_per_step_per_gpu"] = n_pairs
     if args.noise_floor:
@@ -828,25 +879,9 @@ def main():
         line["other_forms"] = forms
 
     def gpu_error(pick, bins, sub, ref):
-        """The GPU's 2F on the CPU baseline's sample (the same bins, signals
-        added by the oracle), chosen form and plain FP32 form, against the
-        oracle's all-core run."""
-        import dataclasses
-        wl = dataclasses.replace(w, bank=sub)
-        out = {}
-        for name, form, algo, tiles in (("chosen", args.form, args.algo, True), ("plain_fp32", "c64", "direct", False)):
-            g3 = fs.FStat(local_rank, dterms=w.dterms, topk=10, bins_form=form, algo=algo,
-                          tile_m=args.tile_m if tiles else 0, tile_warps=args.tile_warps if tiles else 0,
-                          sft_chunk=args.sft_chunk if tiles else 0)
-            try:
-                g3.load_workload(wl, bins_override=bins)
-                g3.compute(stream)
-                got = g3.twoF()
-                st = twoF_error_stats(got, ref)
-                st["variant"] = g3.plan()["variant"]
-                out[name] = st
-            finally:
-                g3.close()
+        out = gpu_2f_error(w, pick, bins, sub, ref, local_rank, stream, bins_form=args.form, algo=args.algo,
+                           tile_m=args.tile_m, tile_warps=args.tile_warps, sft_chunk=args.sft_chunk)
+        out["chosen"]["is_timed_kernel"] = out["chosen"]["kernel"] == kernel_name
         return out
 
     if world == 1 and not args.no_cpu_baseline:

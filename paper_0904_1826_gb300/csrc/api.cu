@@ -573,10 +573,12 @@ int choose_tc(fstat_ctx* c, int P, int L, bool found, Plan& pl, cudaStream_t s) 
     const long long colb = (n_col + kTcCols - 1) / kTcCols;
     const int sms = current_sm_count();
     // Measured on GB300: a block takes 1.44 us an SFT for a tile of 128 x 64
-    // templates, whatever part of it is filled, and the blocks share the steps evenly; the
-    // other forms 5.6e11 pairs/s on
-    // large banks of three or more spindowns, 4.6e11 on one or two, and 2.7e11
-    // where the steps are 1/8 bin (L = 1); smaller banks leave them slower.
+    // templates (1.5 to 1.8 where its windows span four position groups), whatever part
+    // of it is filled, and the blocks share the steps evenly; the other forms 5.6e11
+    // pairs/s on large banks of three or more spindowns, 4.6e11 on one or two, and
+    // 2.7e11 where the steps are 1/8 bin (L = 1).  Smaller banks leave both slower, and
+    // near the line they are level: 48 sky x 1800 f x 3 x 2400, kept on the ring, 1.59
+    // ms there and 1.62 here.
     auto t_tc = [&](int rt) {
         const long long items = ((n_rows + rt - 1) / rt) * colb;
         return (double)items * c->n_sft / tc_blocks((int)((n_rows + rt - 1) / rt), (int)colb, c->n_sft, sms) * 1.44e-6;

@@ -43,9 +43,9 @@
 // integer: about 64 eps of the (row, SFT)) has the two taps by which the windows
 // differ added by the copying warp into a per-block scratch of Fa, Fb.
 //
-// Bound: instruction issue (56 % active, 6750 warp instructions an SFT of 8192
-// pairs: 40 % sums, 40 % weights) with the latency of the stages; tensor pipe
-// 21 %, FMA pipes 43 %.  Against the sinc ring: 4000 sky x 1800 f x 10 spindowns x
+// Bound: instruction issue (61 % of the active cycles, 6810 warp instructions an SFT
+// of 8192 pairs: 40 % sums, 40 % weights) with the latency of the stages; tensor pipe
+// 23 %, FMA pipes 45 %.  Against the sinc ring: 4000 sky x 1800 f x 10 spindowns x
 // 2400 SFTs 203 ms (8.5e11 pairs/s) against 293; 250 x 1733 x 7 x 2302, FP16 bins,
 // 217 Hz 9.1 against 15.7 ms; 2048 x 900 x 1 x 1600 4.1 against 6.9; the 1/8-bin
 // patch 2048 x 256 2.1 against 3.1.

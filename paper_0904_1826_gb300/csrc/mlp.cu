@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(1024) colsum_kernel(const float* __restrict__ 
     if (threadIdx.x < 32 && n < H) out[n] = a;
 }
 
-// All parameters in one launch: the parameter arrays end to end, n[5] the total.
+// All parameters in one launch: the parameter arrays end to end, end[5] the total.
 struct AdamArrays {
     float *p[6], *m[6], *v[6];
     const float* g[6];

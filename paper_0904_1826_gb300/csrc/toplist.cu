@@ -21,7 +21,7 @@
 // Bound: reading the values (HBM) for large banks, group_max at 6.4 TB/s; the
 // launches for small ones.  Whole list, against a radix select with one-thread
 // scans of its histograms and five passes over the values: 60 M values, K = 1000
-// 96 us (624 before); 1.8 M 55 us (152); 800 values, K = 20 11 us (168).  All
+// 96 us (586 before); 1.8 M 55 us (152); 800 values, K = 20 11 us (168).  All
 // values equal, 60 M: 426 us (549).
 #include "fstat_internal.cuh"
 

@@ -124,7 +124,9 @@ typedef struct {
  *   cores instead where the planner finds that faster: window sums from FP16
  *   pairs of bins and weights with FP32 accumulation, closer to the exact sum
  *   than SINCPOLY; in the last bits its results depend on which sky points
- *   share a tile, so on the sky list.  It is kept to SFTs whose largest
+ *   share a tile, so on the sky list and on the number of SMs (SINCPOLY's do
+ *   not: ask for it where the parts of a divided search have to agree to the
+ *   bit with the whole).  It is kept to SFTs whose largest
  *   component, among the bins that the bank's windows reach, is at most 65536
  *   times that of their quietest 16 bins in a row (all-zero ones left out, a
  *   few at the band's edge allowed for):

@@ -1,6 +1,9 @@
 """Host-side pieces of the multi-GPU path: templates shard by sky point with
 no data-path communication; the one exchange is the merge of the per-rank
-toplists (each rank's K best, K x 12 bytes)."""
+toplists (each rank's K best, K x 12 bytes).  The merged list is that of one
+process up to near-ties; it is the same to the bit where the ranks' contexts ask
+for algo="sincpoly" or "direct", as the tensor-core form that "auto" takes on
+large banks groups neighbouring sky points, so its last bits depend on the shard."""
 from __future__ import annotations
 
 import numpy as np

@@ -559,8 +559,8 @@ int tc_range(fstat_ctx* c, cudaStream_t s, bool* fits, int* lo, int* hi) {
 
 // Tensor-core form where it is the faster one.  It needs column steps of one
 // bin (n_sub = P / L templates a bin), a uniform spindown grid, at least 8 SFTs
-// (its blocks work up to 6 ahead) and windows of a tile's rows within
-// kTcMaxSpread bins, and bins of a range that its tables hold (tc_range); Kahan
+// (its blocks work up to 6 ahead), windows of a tile's rows within
+// kTcMaxSpread bins and bins of a range that its tables hold (tc_range); Kahan
 // sums, other D and explicit tile or form requests keep the other forms.
 int choose_tc(fstat_ctx* c, int P, int L, bool found, Plan& pl, cudaStream_t s) {
     pl.tc = pl.tc_by_range = false;
@@ -628,11 +628,10 @@ bool far_eligible(const fstat_ctx* c) {
     return c->opts.dterms == 8 && !c->opts.kahan && c->opts.algo != FSTAT_ALGO_DIRECT;
 }
 
-// Extent of the far-field tables such that every block's rows [x0, x0 + w_pairs)
-// lie inside them: khat is bounded over the bank by the frequency and spindown
-// ranges, |tdot - 1| <= 1.1e-4 (orbital + rotational speed over c) and dtau
-// within the SFT span of t_ref widened by 500 s of Roemer delay.
-// First and last bin, from k_lo, of any window of the bank.
+// First and last bin, from k_lo, of any window of the bank: khat is bounded over
+// it by the frequency and spindown ranges, |tdot - 1| <= 1.1e-4 (orbital +
+// rotational speed over c) and dtau within the SFT span of t_ref widened by 500 s
+// of Roemer delay.
 void bank_reach(const fstat_ctx* c, long long* lo, long long* hi) {
     double tmin = 1e300, tmax = -1e300;
     for (int d = 0; d < kMaxDet; ++d)
@@ -662,6 +661,8 @@ void bank_reach(const fstat_ctx* c, long long* lo, long long* hi) {
     *hi = (long long)std::floor(kmax) - c->k_lo + 8 + 2;
 }
 
+// Extent of the far-field tables such that every block's rows [x0, x0 + w_pairs)
+// lie inside them.
 void far_extent(const fstat_ctx* c, int w_pairs, int* xoff, int* n_pos) {
     long long lo_min, hi_max;
     bank_reach(c, &lo_min, &hi_max);
